@@ -75,7 +75,9 @@ cudaError_t launch_one(ps_plan_s* p, const void* rho, void* V, double* E, cudaSt
 double solve_cost(const ps_plan_s* p) {
   auto f = [&](int j, int N) -> double {
     if (N < 2) return 0.0;
-    const int M = p->blue[j].M;
+    bool tiled = false;  // the tile kernels need no convolution
+    for (int k = 0; k < 5; ++k) tiled |= pass_axis(p, k) == j && p->tile[k].on;
+    const int M = tiled ? 0 : p->blue[j].M;
     return M ? 2.0 * M * std::log2((double)M) + 3.0 * N : N * std::log2((double)N);
   };
   const double n2 = p->n[1], n3 = p->n[2];

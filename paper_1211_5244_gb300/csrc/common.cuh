@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "psolver.h"
+#include "tile_args.cuh"
 
 namespace ps {
 
@@ -164,6 +165,7 @@ struct ps_plan_s {
   ps::Stages st[3];     // stages of the 1D transform per axis (x: length L1/2 if L1 even)
   ps::BlueArgs blue[3]; // Bluestein descriptors per axis (M = 0: off); device pointers owned
   ps::PassCfg cfg[5];
+  ps::TileLaunch tile[5];  // the tile kernels of the passes without a specialised kernel (on = 0: none)
   // fused x/y passes (thread-block clusters): xyf[0] runs passes 1 and 2,
   // xyf[1] passes 4 and 5, when xyfuse is set and rho and V are 16-byte aligned
   int xyfuse;

@@ -573,11 +573,13 @@ cudaError_t configure_passes(ps_plan_s* p) {
       if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget)) != cudaSuccess)
         return e;
   }
+  if ((e = configure_tile<T>(p)) != cudaSuccess) return e;
+  const int tile_parts = p->tile[P3].on ? (int)(p->tile[P3].grid.x * p->tile[P3].grid.y) : 0;
   p->fastord = 0;
   if (!canonical_order(p)) {
     // the generic kernels along strided axes (passes_ord.cu); energy
     // partials: one per CTA of the fused pass
-    p->npart = ord_conv_ctas(p);
+    p->npart = std::max(ord_conv_ctas(p), tile_parts);
     if ((e = configure_ord<T>(p)) != cudaSuccess) return e;
     if constexpr (sizeof(T) == 4) {
       // x first (x, z, y): the specialised x kernels, and the y- and z-pass
@@ -599,7 +601,7 @@ cudaError_t configure_passes(ps_plan_s* p) {
   }
   // energy partials: one per CTA of the z pass
   const int ntk = (p->c + p->cfg[P3].tk - 1) / p->cfg[P3].tk;
-  p->npart = ntk * p->L[1];
+  p->npart = std::max(ntk * p->L[1], tile_parts);
   return cudaSuccess;
 }
 
@@ -634,6 +636,7 @@ cudaError_t launch_solve(ps_plan_s* p, const T* rho, T* V, double* E, cudaStream
   };
   auto pass3 = [&]() -> cudaError_t {
     if (p->cfg[P3].fast) return launch_fast(p, P3, B, B, Ez, escale, s);
+    if (p->tile[P3].on) return launch_tile(p, P3, B, B, E, s);
     GenArgs a = gen_args<T>(p, P3);
     dim3 g((p->c + a.tk - 1) / a.tk, p->L[1]);
     gen_kernels<T>(p->cfg[P3].bm).pz<<<g, p->cfg[P3].threads, p->cfg[P3].gsmem, s>>>(
@@ -670,6 +673,8 @@ cudaError_t launch_solve(ps_plan_s* p, const T* rho, T* V, double* E, cudaStream
     if ((e = launch_xy(p, 0, rho, B, s)) != cudaSuccess) return e;
   } else if (p->cfg[P1].fast && a8) {
     if ((e = launch_fast(p, P1, rho, A, nullptr, 0.0, s)) != cudaSuccess) return e;
+  } else if (p->tile[P1].on) {
+    if ((e = launch_tile(p, P1, rho, A, nullptr, s)) != cudaSuccess) return e;
   } else {
     GenArgs a = gen_args<T>(p, P1);
     const int rpc = (p->L[0] % 2 == 0) ? a.tk : 2 * a.tk;  // odd L1: two real rows per line
@@ -682,6 +687,8 @@ cudaError_t launch_solve(ps_plan_s* p, const T* rho, T* V, double* E, cudaStream
     // done by the fused kernel above
   } else if (p->cfg[P2].fast) {
     if ((e = launch_fast(p, P2, A, B, nullptr, 0.0, s)) != cudaSuccess) return e;
+  } else if (p->tile[P2].on) {
+    if ((e = launch_tile(p, P2, A, B, nullptr, s)) != cudaSuccess) return e;
   } else {
     GenArgs a = gen_args<T>(p, P2);
     dim3 g((p->c + a.tk - 1) / a.tk, p->n[2]);
@@ -696,6 +703,8 @@ cudaError_t launch_solve(ps_plan_s* p, const T* rho, T* V, double* E, cudaStream
     if ((e = launch_xy(p, 1, B, V, s)) != cudaSuccess) return e;
   } else if (p->cfg[P4].fast) {
     if ((e = launch_fast(p, P4, B, A, nullptr, 0.0, s)) != cudaSuccess) return e;
+  } else if (p->tile[P4].on) {
+    if ((e = launch_tile(p, P4, B, A, nullptr, s)) != cudaSuccess) return e;
   } else {
     GenArgs a = gen_args<T>(p, P4);
     dim3 g((p->c + a.tk - 1) / a.tk, p->n[2]);
@@ -707,6 +716,8 @@ cudaError_t launch_solve(ps_plan_s* p, const T* rho, T* V, double* E, cudaStream
     // done by the fused kernel above
   } else if (p->cfg[P5].fast && a8) {
     if ((e = launch_fast(p, P5, A, V, nullptr, 0.0, s)) != cudaSuccess) return e;
+  } else if (p->tile[P5].on) {
+    if ((e = launch_tile(p, P5, A, V, nullptr, s)) != cudaSuccess) return e;
   } else {
     GenArgs a = gen_args<T>(p, P5);
     const int rpc = (p->L[0] % 2 == 0) ? a.tk : 2 * a.tk;  // odd L1: two real rows per line

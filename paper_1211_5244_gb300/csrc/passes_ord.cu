@@ -352,31 +352,41 @@ cudaError_t launch_solve_ord(ps_plan_s* p, const T* rho, T* V, double* E, cudaSt
   cudaError_t e;
   dim3 g;
   if (ev) cudaEventRecord(ev[0], s);
-  if (xfirst) {
+  if (p->tile[P1].on) {
+    if ((e = launch_tile(p, P1, rho, A, nullptr, s)) != cudaSuccess) return e;
+  } else if (xfirst) {
     if ((e = launch_x_pass<T>(p, P1, rho, A, s)) != cudaSuccess) return e;
   } else {
     OrdArgs a = ord_args<T>(p, P1, &g);
     ord_r2c<T><<<g, p->cfg[P1].threads, p->cfg[P1].gsmem, s>>>(rho, A, tw(P1), a);
   }
   if (ev) cudaEventRecord(ev[1], s);
-  {
+  if (p->tile[P2].on) {
+    if ((e = launch_tile(p, P2, A, B, nullptr, s)) != cudaSuccess) return e;
+  } else {
     OrdArgs a = ord_args<T>(p, P2, &g);
     ord_line<-1, T><<<g, p->cfg[P2].threads, p->cfg[P2].gsmem, s>>>(A, B, tw(P2), a);
   }
   if (ev) cudaEventRecord(ev[2], s);
-  {
+  if (p->tile[P3].on) {
+    if ((e = launch_tile(p, P3, B, B, E, s)) != cudaSuccess) return e;
+  } else {
     OrdArgs a = ord_args<T>(p, P3, &g);
     ord_conv<T><<<g, p->cfg[P3].threads, p->cfg[P3].gsmem, s>>>(B, static_cast<const T*>(p->K), tw(P3), a,
                                                                 p->partials, p->counter,
                                                                 0.5 * p->h * p->h * p->h, E);
   }
   if (ev) cudaEventRecord(ev[3], s);
-  {
+  if (p->tile[P4].on) {
+    if ((e = launch_tile(p, P4, B, A, nullptr, s)) != cudaSuccess) return e;
+  } else {
     OrdArgs a = ord_args<T>(p, P4, &g);
     ord_line<1, T><<<g, p->cfg[P4].threads, p->cfg[P4].gsmem, s>>>(B, A, tw(P4), a);
   }
   if (ev) cudaEventRecord(ev[4], s);
-  if (xfirst) {
+  if (p->tile[P5].on) {
+    if ((e = launch_tile(p, P5, A, V, nullptr, s)) != cudaSuccess) return e;
+  } else if (xfirst) {
     if ((e = launch_x_pass<T>(p, P5, A, V, s)) != cudaSuccess) return e;
   } else {
     OrdArgs a = ord_args<T>(p, P5, &g);

@@ -1,0 +1,20 @@
+// Instances of the fused forward, K^F, inverse tile kernels.
+#include "tile_pass.cuh"
+
+namespace ps {
+
+namespace {
+template <bool HALF>
+const void* pick(int cls) {
+  using tile::k_tile_conv;
+  return cls == 0 ? (const void*)k_tile_conv<double, HALF, 0>
+                  : (const void*)k_tile_conv<double, HALF, 1>;
+}
+}  // namespace
+
+template <>
+const void* tile_conv_kernel<double>(bool half, int cls) {
+  return half ? pick<true>(cls) : pick<false>(cls);
+}
+
+}  // namespace ps

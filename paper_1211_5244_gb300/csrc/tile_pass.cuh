@@ -1,0 +1,521 @@
+// Tile kernels: the passes of a solve for any line length with factors up to
+// 13, FP32 and FP64, along any axis, as two (or three) register DFT steps with
+// one exchange through shared memory between them.
+//
+// A CTA owns a tile of tk lines; T threads share a line. With
+// N = Ra Rm Rl, n = n1 NRa + n2 Rl + n3 and k = k1 + Ra k2 + Ra Rm k3 the forward
+// transform is
+//   first  (n2, n3): Ra-point DFT over n1 -> k1, inputs straight from global memory
+//   middle (k1, n3): inputs times W_N^{k1 Rl n2}, Rm-point DFT over n2 -> k2
+//   last   (k1, k2): inputs times W_N^{(k1 + Ra k2) n3}, Rl-point DFT over n3 -> k3,
+//                    outputs straight to global memory at k1 + Ra k2 + Ra Rm k3
+// and the inverse the same steps backwards (twiddles before the middle and the
+// final step). Every step replaces the tile elements it read, so one buffer
+// serves all of them; the fused pass multiplies by K^F between the last forward
+// and the first inverse step, which share their elements, in registers.
+//
+// What bounds them: in FP32 issue and latency (100 x 90 x 110 free, L = 200 x 180 x
+// 220: 250 -> 63 us per solve against the Stockham and Bluestein kernels of
+// passes.cu, which make a shared-memory round trip per stage and more for the load,
+// the multiply and the store, and spend a third of their issue slots on integer
+// instructions), in FP64 the two FP64 lanes per clock and SM (128^3 free: 1657
+// -> 1215 us; the pipe was 84% busy before, so only fewer operations help).
+#pragma once
+
+#include "fft_fast.cuh"
+#include "tile_dft.cuh"
+
+namespace ps {
+namespace tile {
+
+// calls f(integral_constant<R>) for the run-time radix R of a step
+template <int CLS, class F>
+__device__ __forceinline__ void radix_switch(int R, F&& f) {
+#define PS_RADIX(r) \
+  case r: f(std::integral_constant<int, r>{}); break;
+  if constexpr (CLS == 0) {
+    switch (R) {
+      PS_RADIX(2) PS_RADIX(3) PS_RADIX(4) PS_RADIX(5) PS_RADIX(6) PS_RADIX(7) PS_RADIX(8)
+      default: break;
+    }
+  } else {
+    switch (R) {
+      PS_RADIX(2) PS_RADIX(3) PS_RADIX(4) PS_RADIX(5) PS_RADIX(6) PS_RADIX(7) PS_RADIX(8) PS_RADIX(9)
+      PS_RADIX(10) PS_RADIX(11) PS_RADIX(12) PS_RADIX(13) PS_RADIX(14) PS_RADIX(15) PS_RADIX(16)
+      default: break;
+    }
+  }
+#undef PS_RADIX
+}
+
+// The tile: lines [t * ls] of elements in shared memory, the table W_N^j after them.
+template <class C>
+struct Tile {
+  C* sh;
+  const C* tw;
+};
+
+// the tile's place, and the asynchronous copy of the twiddle table, which the
+// first step does not read: steps_sync after it
+template <class C>
+__device__ __forceinline__ Tile<C> tile_setup(const TileArgs& a, unsigned char* raw) {
+  Tile<C> s;
+  s.sh = reinterpret_cast<C*>(raw);
+  C* tw = s.sh + a.elems;
+  const C* g = static_cast<const C*>(a.tw);
+  for (int i = threadIdx.x; i < a.N; i += blockDim.x) {
+    if constexpr (sizeof(C) == 8)
+      cp_async8(tw + i, g + (long long)i * a.tws);
+    else
+      cp_async16(tw + i, g + (long long)i * a.tws);
+  }
+  cp_async_commit();
+  s.tw = tw;
+  return s;
+}
+__device__ __forceinline__ void steps_sync() {
+  cp_async_wait_all();
+  __syncthreads();
+}
+
+// calls f(t, b) for this thread's share of the nb butterflies of each of the
+// tile's tk lines: consecutive threads along the lines' butterflies where the
+// lines are the contiguous axis, else across the lines. No thread idles but in
+// the last round, whatever nb is (an idle lane costs as much FP64 time as a busy one).
+template <class F>
+__device__ __forceinline__ void tasks(const TileArgs& a, int nb, unsigned mnb, F&& f) {
+  const int n = nb << a.ltk;
+  for (int w = threadIdx.x; w < n; w += blockDim.x) {
+    int t, b;
+    if (a.lc) {
+      t = div_by(w, mnb);
+      b = w - t * nb;
+    } else {
+      t = w & (a.tk - 1);
+      b = w >> a.ltk;
+    }
+    f(t, b);
+  }
+}
+
+// The tile's line t: its index along the tile axis and its plane; false beyond
+// the last one. Tiles belong to one plane (blockIdx.y), or run over the lines of
+// all planes in sequence (flat), so that only the last tile is ragged.
+__device__ __forceinline__ bool line_of(const TileArgs& a, int t, int* line, int* pl) {
+  const unsigned g = blockIdx.x * (unsigned)a.tk + t;
+  if (!a.flat) {
+    *line = (int)g;
+    *pl = blockIdx.y;
+    return g < (unsigned)a.ntl;
+  }
+  const unsigned p = g / (unsigned)a.ntl;
+  *line = (int)(g - p * (unsigned)a.ntl);
+  *pl = (int)p;
+  return p < (unsigned)a.npl;
+}
+
+// tile position and exponent (k1 + Ra k2) of butterfly bf of the last step
+__device__ __forceinline__ void last_digits(const TileArgs& a, int bf, int* pos, int* e) {
+  if (a.Rm == 1) {
+    *pos = bf * a.s1;
+    *e = bf;
+  } else {
+    const int k1 = div_by(bf, a.mRm), k2 = bf - k1 * a.Rm;
+    *pos = k1 * a.s1 + k2 * a.s2;
+    *e = k1 + a.Ra * k2;
+  }
+}
+// tile position of output k after the last forward step
+__device__ __forceinline__ int k_pos(const TileArgs& a, int k) {
+  const int q = div_by(k, a.mRa), k1 = k - q * a.Ra;
+  if (a.Rm == 1) return k1 * a.s1 + q * a.es;
+  const int r = div_by(q, a.mRm), k2 = q - r * a.Rm;
+  return k1 * a.s1 + k2 * a.s2 + r * a.es;
+}
+
+// first forward step: lines(t)(element) gives the inputs, half of them zero for HALF
+template <int DIR, bool HALF, int CLS, class C, class Ln>
+__device__ __forceinline__ void step_first(const TileArgs& a, const Tile<C>& s, Ln&& lines) {
+  radix_switch<CLS>(a.Ra, [&](auto rc) {
+    constexpr int R = rc;
+    if constexpr (!HALF || R % 2 == 0) {
+      constexpr int RN = HALF ? R / 2 : R;
+      tasks(a, a.NRa, a.mNRa, [&](int t, int b) {
+        const auto ld = lines(t);
+        C x[R];
+#pragma unroll
+        for (int r = 0; r < RN; ++r) x[r] = ld(b + r * a.NRa);
+        dft<R, DIR, full_mask(RN)>(x);
+        C* p = s.sh + t * a.ls + b * a.es;
+#pragma unroll
+        for (int r = 0; r < R; ++r) p[r * a.s1] = x[r];
+      });
+    }
+  });
+}
+// final inverse step: lines(t)(element, value) takes the outputs, the lower half for HALF
+template <bool HALF, int CLS, class C, class Ln>
+__device__ __forceinline__ void step_final(const TileArgs& a, const Tile<C>& s, Ln&& lines) {
+  radix_switch<CLS>(a.Ra, [&](auto rc) {
+    constexpr int R = rc;
+    if constexpr (!HALF || R % 2 == 0) {
+      constexpr int RN = HALF ? R / 2 : R;
+      tasks(a, a.NRa, a.mNRa, [&](int t, int b) {
+        C x[R];
+        const C* p = s.sh + t * a.ls + b * a.es;
+#pragma unroll
+        for (int r = 0; r < R; ++r) x[r] = p[r * a.s1];
+        dft_pre<R, 1>(x, s.tw, b, a.NRa);
+        const auto st = lines(t);
+#pragma unroll
+        for (int r = 0; r < RN; ++r) st(b + r * a.NRa, x[r]);
+      });
+    }
+  });
+}
+// middle step of three, in place
+template <int DIR, int CLS, class C>
+__device__ __forceinline__ void step_middle(const TileArgs& a, const Tile<C>& s) {
+  if (a.Rm == 1) return;
+  const int NRm = a.Ra * a.Rl;
+  radix_switch<CLS>(a.Rm, [&](auto rc) {
+    constexpr int R = rc;
+    tasks(a, NRm, a.mNRm, [&](int t, int b) {
+      const int k1 = div_by(b, a.mRl), n3 = b - k1 * a.Rl;
+      C* p = s.sh + t * a.ls + k1 * a.s1 + n3 * a.es;
+      C x[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) x[r] = p[r * a.s2];
+      dft_pre<R, DIR>(x, s.tw, DIR < 0 ? k1 * a.Rl : a.Ra * n3, NRm);
+#pragma unroll
+      for (int r = 0; r < R; ++r) p[r * a.s2] = x[r];
+    });
+  });
+  __syncthreads();
+}
+// last forward step: lines(t)(tile address, k, value) takes the outputs
+template <int CLS, class C, class Ln>
+__device__ __forceinline__ void step_last(const TileArgs& a, const Tile<C>& s, Ln&& lines) {
+  radix_switch<CLS>(a.Rl, [&](auto rc) {
+    constexpr int R = rc;
+    tasks(a, a.Kl, a.mKl, [&](int t, int b) {
+      int pos, e;
+      last_digits(a, b, &pos, &e);
+      C* p = s.sh + t * a.ls + pos;
+      C x[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) x[r] = p[r * a.es];
+      dft_pre<R, -1>(x, s.tw, e, a.Kl);
+      const auto st = lines(t);
+#pragma unroll
+      for (int r = 0; r < R; ++r) st(p + r * a.es, e + r * a.Kl, x[r]);
+    });
+  });
+}
+// first inverse step: lines(t)(tile address, k) gives the inputs
+template <int CLS, class C, class Ln>
+__device__ __forceinline__ void step_inv_first(const TileArgs& a, const Tile<C>& s, Ln&& lines) {
+  radix_switch<CLS>(a.Rl, [&](auto rc) {
+    constexpr int R = rc;
+    tasks(a, a.Kl, a.mKl, [&](int t, int b) {
+      const auto ld = lines(t);
+      int pos, e;
+      last_digits(a, b, &pos, &e);
+      C* p = s.sh + t * a.ls + pos;
+      C x[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) x[r] = ld(p + r * a.es, e + r * a.Kl);
+      dft<R, 1, full_mask(R)>(x);
+#pragma unroll
+      for (int r = 0; r < R; ++r) p[r * a.es] = x[r];
+    });
+  });
+}
+
+template <typename T, int CLS>
+struct Bounds {  // resident CTAs per SM asked of the compiler
+  static constexpr int per_sm = sizeof(T) == 4 ? (CLS == 0 ? 4 : 3) : (CLS == 0 ? 3 : 2);
+};
+
+// ------------------------------------------------------------ complex lines
+
+// DIR -1: nin inputs (the rest zero), N outputs; +1: N inputs, nout outputs
+template <typename T, int DIR, bool HALF, int CLS>
+__global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_line(const __grid_constant__ TileArgs a) {
+  using C = cpx<T>;
+  extern __shared__ __align__(16) unsigned char raw[];
+  const Tile<C> s = tile_setup<C>(a, raw);
+  // the lines of the tile at their source and destination
+  auto in = [&](int t, bool* ok) {
+    int line, pl;
+    *ok = line_of(a, t, &line, &pl);
+    return static_cast<const C*>(a.src) + (pl * a.sp_in + line * a.st_in);
+  };
+  auto out = [&](int t, bool* ok) {
+    int line, pl;
+    *ok = line_of(a, t, &line, &pl);
+    return static_cast<C*>(a.dst) + (pl * a.sp_out + line * a.st_out);
+  };
+  pdl_wait();
+  if constexpr (DIR < 0) {
+    step_first<-1, HALF, CLS>(a, s, [&](int t) {
+      bool ok;
+      const C* src = in(t, &ok);
+      return [&a, src, ok](int e) { return ok && e < a.nin ? src[(long long)e * a.se_in] : mk(T(0), T(0)); };
+    });
+    steps_sync();
+    step_middle<-1, CLS>(a, s);
+    step_last<CLS>(a, s, [&](int t) {
+      bool ok;
+      C* dst = out(t, &ok);
+      return [&a, dst, ok](C*, int k, C v) {
+        if (ok) dst[(long long)k * a.se_out] = v;
+      };
+    });
+  } else {
+    step_inv_first<CLS>(a, s, [&](int t) {
+      bool ok;
+      const C* src = in(t, &ok);
+      return [&a, src, ok](C*, int k) { return ok ? src[(long long)k * a.se_in] : mk(T(0), T(0)); };
+    });
+    steps_sync();
+    step_middle<1, CLS>(a, s);
+    step_final<HALF, CLS>(a, s, [&](int t) {
+      bool ok;
+      C* dst = out(t, &ok);
+      return [&a, dst, ok](int e, C v) {
+        if (ok && e < a.nout) dst[(long long)e * a.se_out] = v;
+      };
+    });
+  }
+}
+
+// ------------------------------------------------------------ forward, K^F, inverse
+
+// The energy of the fused pass, in two halves around the inverse transform so
+// that its fence and atomic run beside it instead of holding every CTA at its end
+// (L = 220, 18180 lines on 2273 CTAs: 47.3 us with the reduction at the end).
+// Before a barrier: the warp sums. After it: energy_arrive in thread 0 adds
+// them, stores the CTA's partial and counts its arrival. At the end the first warp of
+// the CTA that arrived last adds all partials in index order and resets the counter.
+template <typename T>
+__device__ __forceinline__ void energy_warps(T en, T* wsum) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) en += __shfl_xor_sync(0xffffffffu, en, o);
+  if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = en;
+}
+template <typename T>
+__device__ __forceinline__ unsigned energy_arrive(const TileArgs& a, const T* wsum) {
+  double sum = 0.0;
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) sum += (double)wsum[w];
+  a.partials[blockIdx.y * gridDim.x + blockIdx.x] = sum;
+  __threadfence();
+  return atomicAdd(a.counter, 1u);
+}
+__device__ __forceinline__ void energy_last(const TileArgs& a, unsigned arrived) {
+  const unsigned n = gridDim.x * gridDim.y;
+  if (__shfl_sync(0xffffffffu, arrived, 0) != n - 1) return;
+  __threadfence();
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  for (unsigned i = threadIdx.x; i < n; i += 128)
+#pragma unroll
+    for (unsigned u = 0; u < 4; ++u)
+      if (i + 32 * u < n) acc[u] += __ldcg(a.partials + i + 32 * u);
+  double sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if (threadIdx.x == 0) {
+    *a.E = a.escale * sum;
+    *a.counter = 0u;
+  }
+}
+
+template <typename T, bool HALF, int CLS>
+__global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_conv(const __grid_constant__ TileArgs a) {
+  using C = cpx<T>;
+  extern __shared__ __align__(16) unsigned char raw[];
+  __shared__ T wsum[8];
+  const Tile<C> s = tile_setup<C>(a, raw);
+  auto at = [&](int t, int* line, int* pl) {
+    const bool ok = line_of(a, t, line, pl);
+    if (a.pair_pl && ok) *pl = paired_ky(*pl, a.npl);
+    return ok;
+  };
+  auto ptr = [&](int t, bool* ok) {
+    int line, pl;
+    *ok = at(t, &line, &pl);
+    return static_cast<C*>(a.dst) + (pl * a.sp_in + line * a.st_in);
+  };
+  pdl_wait();
+  step_first<-1, HALF, CLS>(a, s, [&](int t) {
+    bool ok;
+    const C* src = ptr(t, &ok);
+    return [&a, src, ok](int e) { return ok && e < a.nin ? src[(long long)e * a.se_in] : mk(T(0), T(0)); };
+  });
+  steps_sync();
+  step_middle<-1, CLS>(a, s);
+  T en = T(0);
+  radix_switch<CLS>(a.Rl, [&](auto rc) {
+    constexpr int R = rc;
+    tasks(a, a.Kl, a.mKl, [&](int t, int b) {
+      int line, pl, pos, e;
+      const bool ok = at(t, &line, &pl);
+      const T* Kp = static_cast<const T*>(a.K) + (long long)min(pl, a.Lp - pl) * a.Ksp +
+                    (long long)min(line, a.Lt - line) * a.Kst;
+      last_digits(a, b, &pos, &e);
+      T kk[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int k = e + r * a.Kl;
+        kk[r] = ok ? __ldg(Kp + (long long)min(k, a.N - k) * a.Kse) : T(0);
+      }
+      C* p = s.sh + t * a.ls + pos;
+      C x[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) x[r] = p[r * a.es];
+      dft_pre<R, -1>(x, s.tw, e, a.Kl);
+      T el = T(0);
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const C u = mk(kk[r] * x[r].x, kk[r] * x[r].y);
+        el = mad(u.x, x[r].x, mad(u.y, x[r].y, el));  // K |rho^F|^2
+        x[r] = u;
+      }
+      const int k0 = a.w_tile ? line : pl;
+      en = mad(k0 == 0 || 2 * k0 == a.La0 ? T(1) : T(2), el, en);
+      dft<R, 1, full_mask(R)>(x);
+#pragma unroll
+      for (int r = 0; r < R; ++r) p[r * a.es] = x[r];
+    });
+  });
+  if (a.E != nullptr) energy_warps(en, wsum);
+  __syncthreads();
+  unsigned arrived = 0;
+  if (a.E != nullptr && threadIdx.x == 0) arrived = energy_arrive(a, wsum);
+  step_middle<1, CLS>(a, s);
+  step_final<HALF, CLS>(a, s, [&](int t) {
+    bool ok;
+    C* dst = ptr(t, &ok);
+    return [&a, dst, ok](int e, C v) {
+      if (ok && e < a.nout) dst[(long long)e * a.se_out] = v;
+    };
+  });
+  if (a.E != nullptr && threadIdx.x < 32) energy_last(a, arrived);
+}
+
+// ------------------------------------------------------------ real passes
+
+// PAIR: a line is two real sequences a + i b of length N (columns 2t and 2t + 1
+// along y or z, or rows 2t and 2t + 1 of an odd x axis), separated by
+//   A[k] = (Z[k] + conj Z[N-k]) / 2,  B[k] = (Z[k] - conj Z[N-k]) / 2i,  k <= N/2;
+// else a row of length L = 2 N packed as z[m] = x[2m] + i x[2m+1], untangled by
+//   X[k] = E[k] + W_L^k O[k],  E = (Z[k] + conj Z[N-k]) / 2,  O = -i (Z[k] - conj Z[N-k]) / 2.
+// A line of a pair has its second sequence unless it is the last of an odd number.
+template <typename T, bool PAIR, bool HALF, int CLS>
+__global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_r2c(const __grid_constant__ TileArgs a) {
+  using C = cpx<T>;
+  extern __shared__ __align__(16) unsigned char raw[];
+  const Tile<C> s = tile_setup<C>(a, raw);
+  pdl_wait();
+  step_first<-1, HALF, CLS>(a, s, [&](int t) {
+    int line, pl;
+    const bool ok = line_of(a, t, &line, &pl);
+    const T* src = static_cast<const T*>(a.rsrc) + (pl * a.sp_in + line * a.st_in);
+    const bool two = PAIR && 2 * line + 1 < a.nreal;
+    return [&a, src, ok, two](int e) {
+      C v = mk(T(0), T(0));
+      if (!ok || e >= a.nin) return v;
+      const T* p = src + (long long)e * a.se_in;
+      const bool im = PAIR ? two : 2 * e + 1 < a.nreal;
+      if (a.vec && im) return *reinterpret_cast<const C*>(p);
+      v.x = p[0];
+      if (im) v.y = p[a.im_off];
+      return v;
+    };
+  });
+  steps_sync();
+  step_middle<-1, CLS>(a, s);
+  step_last<CLS>(a, s, [&](int) { return [](C* p, int, C v) { *p = v; }; });
+  __syncthreads();
+  const int N = a.N;
+  tasks(a, N / 2 + 1, a.mout, [&](int t, int k) {
+    int line, pl;
+    if (!line_of(a, t, &line, &pl)) return;
+    const C* z = s.sh + t * a.ls;
+    const C zk = z[k_pos(a, k)];
+    const C zm = z[k_pos(a, k == 0 ? 0 : N - k)];
+    const C e = mk(T(0.5) * (zk.x + zm.x), T(0.5) * (zk.y - zm.y));
+    const C o = mk(T(0.5) * (zk.y + zm.y), T(0.5) * (zm.x - zk.x));
+    C* d = static_cast<C*>(a.dst) + (pl * a.sp_out + line * a.st_out);
+    if constexpr (PAIR) {
+      d[(long long)k * a.se_out] = e;
+      if (2 * line + 1 < a.nreal) d[(long long)k * a.se_out + a.im_c] = o;
+    } else {
+      // outputs k and N - k from the same pair: X[N-k] = conj(E - W^k O)
+      const C wo = mul_w<-1>(o, __ldg(static_cast<const C*>(a.twL) + k));
+      d[k] = cadd(e, wo);
+      if (2 * k != N) d[N - k] = mk(e.x - wo.x, wo.y - e.y);
+    }
+  });
+}
+
+template <typename T, bool PAIR, bool HALF, int CLS>
+__global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_c2r(const __grid_constant__ TileArgs a) {
+  using C = cpx<T>;
+  extern __shared__ __align__(16) unsigned char raw[];
+  const Tile<C> s = tile_setup<C>(a, raw);
+  const int N = a.N;
+  pdl_wait();
+  // Z[k] and Z[N-k] from the same pair of inputs
+  tasks(a, N / 2 + 1, a.mout, [&](int t, int k) {
+    int line, pl;
+    C zk = mk(T(0), T(0)), zm = zk;
+    if (line_of(a, t, &line, &pl)) {
+      const C* x = static_cast<const C*>(a.src) + (pl * a.sp_in + line * a.st_in);
+      if constexpr (PAIR) {
+        // Z[k] = A + i B, Z[N-k] = conj A + i conj B; A and B are real at k = 0 and
+        // N/2, so their (rounding-level) imaginary parts there are dropped
+        C A = x[(long long)k * a.se_in], B = zk;
+        if (2 * line + 1 < a.nreal) B = x[(long long)k * a.se_in + a.im_c];
+        if (k == 0 || 2 * k == N) A.y = B.y = T(0);
+        zk = mk(A.x - B.y, A.y + B.x);
+        zm = mk(A.x + B.y, B.x - A.y);
+      } else {
+        // Z[k] = E' + i O', E' = X[k] + conj X[N-k], O' = (X[k] - conj X[N-k]) conj W_L^k;
+        // E'[N-k] = conj E'[k], O'[N-k] = conj O'[k]
+        const C xk = x[k], xm = x[N - k];
+        const C e = mk(xk.x + xm.x, xk.y - xm.y);
+        const C o = mul_w<1>(mk(xk.x - xm.x, xk.y + xm.y), __ldg(static_cast<const C*>(a.twL) + k));
+        zk = mk(e.x - o.y, e.y + o.x);
+        zm = mk(e.x + o.y, o.x - e.y);
+      }
+    }
+    C* z = s.sh + t * a.ls;
+    z[k_pos(a, k)] = zk;
+    if (k != 0 && 2 * k != N) z[k_pos(a, N - k)] = zm;
+  });
+  __syncthreads();
+  step_inv_first<CLS>(a, s, [&](int) { return [](C* p, int) { return *p; }; });
+  steps_sync();
+  step_middle<1, CLS>(a, s);
+  step_final<HALF, CLS>(a, s, [&](int t) {
+    int line, pl;
+    const bool ok = line_of(a, t, &line, &pl);
+    T* dst = static_cast<T*>(a.rdst) + (pl * a.sp_out + line * a.st_out);
+    const bool two = PAIR && 2 * line + 1 < a.nreal;
+    return [&a, dst, ok, two](int e, C v) {
+      if (!ok || e >= a.nout) return;
+      T* p = dst + (long long)e * a.se_out;
+      const bool im = PAIR ? two : 2 * e + 1 < a.nreal;
+      if (a.vec && im) {
+        *reinterpret_cast<C*>(p) = v;
+      } else {
+        p[0] = v.x;
+        if (im) p[a.im_off] = v.y;
+      }
+    };
+  });
+}
+
+}  // namespace tile
+}  // namespace ps

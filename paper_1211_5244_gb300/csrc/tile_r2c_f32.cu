@@ -1,0 +1,21 @@
+// Instances of the real tile kernels (r2c).
+#include "tile_pass.cuh"
+
+namespace ps {
+
+namespace {
+template <bool PAIR, bool HALF>
+const void* pick(int cls) {
+  using tile::k_tile_r2c;
+  return cls == 0 ? (const void*)k_tile_r2c<float, PAIR, HALF, 0>
+                  : (const void*)k_tile_r2c<float, PAIR, HALF, 1>;
+}
+}  // namespace
+
+template <>
+const void* tile_r2c_kernel<float>(bool pair, bool half, int cls) {
+  if (pair) return half ? pick<true, true>(cls) : pick<true, false>(cls);
+  return half ? pick<false, true>(cls) : pick<false, false>(cls);
+}
+
+}  // namespace ps
