@@ -7,8 +7,7 @@ namespace {
 template <bool PAIR, bool HALF>
 const void* pick(int cls) {
   using tile::k_tile_c2r;
-  return cls == 0 ? (const void*)k_tile_c2r<float, PAIR, HALF, 0>
-                  : (const void*)k_tile_c2r<float, PAIR, HALF, 1>;
+  return cls == 0 ? (const void*)k_tile_c2r<float, PAIR, HALF, 0> : cls == 1 ? (const void*)k_tile_c2r<float, PAIR, HALF, 1> : (const void*)k_tile_c2r<float, PAIR, HALF, 2>;
 }
 }  // namespace
 

@@ -7,8 +7,7 @@ namespace {
 template <bool HALF>
 const void* pick(int cls) {
   using tile::k_tile_conv;
-  return cls == 0 ? (const void*)k_tile_conv<float, HALF, 0>
-                  : (const void*)k_tile_conv<float, HALF, 1>;
+  return cls == 0 ? (const void*)k_tile_conv<float, HALF, 0> : cls == 1 ? (const void*)k_tile_conv<float, HALF, 1> : (const void*)k_tile_conv<float, HALF, 2>;
 }
 }  // namespace
 

@@ -43,27 +43,35 @@ double dft_pre_ops(int R) {
 // and larger radices take more registers (0.2 per point). In FP64 the pipe's
 // operations are the time: 256 = 8 x 4 x 8 and 16 x 16 take 224 us each for 10368
 // lines, 200 = 10 x 4 x 5 219 us where 10 x 2 x 10 takes 254.
-// Lengths with a factor of 17 or more stay on the kernels of passes.cu.
+// A length with one prime factor from 17 to 31 takes it as its last radix: about p + 3
+// operations per element, where the Bluestein convolution of passes.cu runs two
+// transforms of at least twice the length.
 bool tile_radix(int N, bool even_first, bool f32, TileRadix* out) {
   constexpr int kMax = 16;
   const double step = f32 ? 2.0 : 0.0;
   auto small = [](int R) { return R == 2 ? 4.0 : 0.0; };
   double best = -1.0;
+  auto consider = [&](int Ra, int Rm, int Rl, int cls) {
+    const int most = std::max(Ra, std::max(Rm, Rl));
+    double c = dft_ops(Ra) / Ra + dft_pre_ops(Rl) / Rl + 2 * step + small(Ra) + small(Rl) + 0.2 * most;
+    if (Rm > 1) c += dft_pre_ops(Rm) / Rm + step + small(Rm);
+    if (best < 0.0 || c < best) {
+      best = c;
+      *out = TileRadix{Ra, Rm, Rl, cls};
+    }
+  };
   for (int Ra = 2; Ra <= kMax; ++Ra) {
     if (N % Ra || (even_first && Ra % 2)) continue;
     const int q = N / Ra;
-    for (int Rl = 2; Rl <= kMax; ++Rl) {
-      if (q % Rl) continue;
-      const int Rm = q / Rl;
-      if (Rm > kMax) continue;
-      const int most = std::max(Ra, std::max(Rm, Rl));
-      double c = dft_ops(Ra) / Ra + dft_pre_ops(Rl) / Rl + 2 * step + small(Ra) + small(Rl) + 0.2 * most;
-      if (Rm > 1) c += dft_pre_ops(Rm) / Rm + step + small(Rm);
-      if (best < 0.0 || c < best) {
-        best = c;
-        *out = TileRadix{Ra, Rm, Rl, most > 8 ? 1 : 0};
-      }
-    }
+    for (int Rl = 2; Rl <= kMax; ++Rl)
+      if (q % Rl == 0 && q / Rl <= kMax) consider(Ra, q / Rl, Rl, std::max(Ra, std::max(q / Rl, Rl)) > 8 ? 1 : 0);
+  }
+  if (best >= 0.0) return true;
+  for (const int p : {17, 19, 23, 29, 31}) {
+    if (N % p) continue;
+    const int q = N / p;
+    for (int Ra = q == 1 ? 1 : 2; Ra <= kMax; ++Ra)
+      if (q % Ra == 0 && q / Ra <= kMax && !(even_first && Ra % 2)) consider(Ra, q / Ra, p, 2);
   }
   return best >= 0.0;
 }
@@ -103,7 +111,7 @@ TileShape pick_tile(const TileArgs& a, const TileRadix& r, int row, long long li
   const double ops[3] = {dft_ops(r.Ra), dft_pre_ops(r.Rl), dft_pre_ops(r.Rm)};
   auto bytes = [&](int tk) { return ((size_t)row * tk + a.N) * csz; };
   int tk = want;
-  if (tk == 0 && f32) tk = a.N <= 160 ? 16 : 8;
+  if (tk == 0 && f32) tk = a.Kl == 1 ? 32 : a.N <= 160 ? 16 : 8;
   if (tk == 0) {
     double best = -1.0;
     for (int v : {8, 16, 32, 4}) {

@@ -7,8 +7,7 @@ namespace {
 template <int DIR, bool HALF>
 const void* pick(int cls) {
   using tile::k_tile_line;
-  return cls == 0 ? (const void*)k_tile_line<double, DIR, HALF, 0>
-                  : (const void*)k_tile_line<double, DIR, HALF, 1>;
+  return cls == 0 ? (const void*)k_tile_line<double, DIR, HALF, 0> : cls == 1 ? (const void*)k_tile_line<double, DIR, HALF, 1> : (const void*)k_tile_line<double, DIR, HALF, 2>;
 }
 }  // namespace
 

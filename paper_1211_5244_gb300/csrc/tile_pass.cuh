@@ -28,8 +28,11 @@
 namespace ps {
 namespace tile {
 
-// calls f(integral_constant<R>) for the run-time radix R of a step
-template <int CLS, class F>
+// calls f(integral_constant<R>) for the run-time radix R of a step. Class 0: radices
+// up to 8, class 1: up to 16, class 2: a prime from 17 to 31 in the last forward
+// (first inverse) step, LAST, and radices up to 16, or 1, in the others. The class
+// bounds a kernel's registers, hence the separate instances.
+template <int CLS, bool LAST, class F>
 __device__ __forceinline__ void radix_switch(int R, F&& f) {
 #define PS_RADIX(r) \
   case r: f(std::integral_constant<int, r>{}); break;
@@ -38,7 +41,15 @@ __device__ __forceinline__ void radix_switch(int R, F&& f) {
       PS_RADIX(2) PS_RADIX(3) PS_RADIX(4) PS_RADIX(5) PS_RADIX(6) PS_RADIX(7) PS_RADIX(8)
       default: break;
     }
+  } else if constexpr (CLS == 2 && LAST) {
+    switch (R) {
+      PS_RADIX(17) PS_RADIX(19) PS_RADIX(23) PS_RADIX(29) PS_RADIX(31)
+      default: break;
+    }
   } else {
+    if constexpr (CLS == 2) {
+      if (R == 1) f(std::integral_constant<int, 1>{});
+    }
     switch (R) {
       PS_RADIX(2) PS_RADIX(3) PS_RADIX(4) PS_RADIX(5) PS_RADIX(6) PS_RADIX(7) PS_RADIX(8) PS_RADIX(9)
       PS_RADIX(10) PS_RADIX(11) PS_RADIX(12) PS_RADIX(13) PS_RADIX(14) PS_RADIX(15) PS_RADIX(16)
@@ -136,7 +147,7 @@ __device__ __forceinline__ int k_pos(const TileArgs& a, int k) {
 // first forward step: lines(t)(element) gives the inputs, half of them zero for HALF
 template <int DIR, bool HALF, int CLS, class C, class Ln>
 __device__ __forceinline__ void step_first(const TileArgs& a, const Tile<C>& s, Ln&& lines) {
-  radix_switch<CLS>(a.Ra, [&](auto rc) {
+  radix_switch<CLS, false>(a.Ra, [&](auto rc) {
     constexpr int R = rc;
     if constexpr (!HALF || R % 2 == 0) {
       constexpr int RN = HALF ? R / 2 : R;
@@ -156,7 +167,7 @@ __device__ __forceinline__ void step_first(const TileArgs& a, const Tile<C>& s, 
 // final inverse step: lines(t)(element, value) takes the outputs, the lower half for HALF
 template <bool HALF, int CLS, class C, class Ln>
 __device__ __forceinline__ void step_final(const TileArgs& a, const Tile<C>& s, Ln&& lines) {
-  radix_switch<CLS>(a.Ra, [&](auto rc) {
+  radix_switch<CLS, false>(a.Ra, [&](auto rc) {
     constexpr int R = rc;
     if constexpr (!HALF || R % 2 == 0) {
       constexpr int RN = HALF ? R / 2 : R;
@@ -178,7 +189,7 @@ template <int DIR, int CLS, class C>
 __device__ __forceinline__ void step_middle(const TileArgs& a, const Tile<C>& s) {
   if (a.Rm == 1) return;
   const int NRm = a.Ra * a.Rl;
-  radix_switch<CLS>(a.Rm, [&](auto rc) {
+  radix_switch<CLS, false>(a.Rm, [&](auto rc) {
     constexpr int R = rc;
     tasks(a, NRm, a.mNRm, [&](int t, int b) {
       const int k1 = div_by(b, a.mRl), n3 = b - k1 * a.Rl;
@@ -196,7 +207,7 @@ __device__ __forceinline__ void step_middle(const TileArgs& a, const Tile<C>& s)
 // last forward step: lines(t)(tile address, k, value) takes the outputs
 template <int CLS, class C, class Ln>
 __device__ __forceinline__ void step_last(const TileArgs& a, const Tile<C>& s, Ln&& lines) {
-  radix_switch<CLS>(a.Rl, [&](auto rc) {
+  radix_switch<CLS, true>(a.Rl, [&](auto rc) {
     constexpr int R = rc;
     tasks(a, a.Kl, a.mKl, [&](int t, int b) {
       int pos, e;
@@ -215,7 +226,7 @@ __device__ __forceinline__ void step_last(const TileArgs& a, const Tile<C>& s, L
 // first inverse step: lines(t)(tile address, k) gives the inputs
 template <int CLS, class C, class Ln>
 __device__ __forceinline__ void step_inv_first(const TileArgs& a, const Tile<C>& s, Ln&& lines) {
-  radix_switch<CLS>(a.Rl, [&](auto rc) {
+  radix_switch<CLS, true>(a.Rl, [&](auto rc) {
     constexpr int R = rc;
     tasks(a, a.Kl, a.mKl, [&](int t, int b) {
       const auto ld = lines(t);
@@ -234,7 +245,7 @@ __device__ __forceinline__ void step_inv_first(const TileArgs& a, const Tile<C>&
 
 template <typename T, int CLS>
 struct Bounds {  // resident CTAs per SM asked of the compiler
-  static constexpr int per_sm = sizeof(T) == 4 ? (CLS == 0 ? 4 : 3) : (CLS == 0 ? 3 : 2);
+  static constexpr int per_sm = sizeof(T) == 4 ? (CLS == 0 ? 4 : CLS == 1 ? 3 : 2) : (CLS == 0 ? 3 : CLS == 1 ? 2 : 1);
 };
 
 // ------------------------------------------------------------ complex lines
@@ -355,7 +366,7 @@ __global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_conv(const
   steps_sync();
   step_middle<-1, CLS>(a, s);
   T en = T(0);
-  radix_switch<CLS>(a.Rl, [&](auto rc) {
+  radix_switch<CLS, true>(a.Rl, [&](auto rc) {
     constexpr int R = rc;
     tasks(a, a.Kl, a.mKl, [&](int t, int b) {
       int line, pl, pos, e;
