@@ -88,6 +88,7 @@ struct FastArgs {
                           // beyond nl are zero on input and not stored on output
   int rev;                // walk the z planes (y passes) or rows (x passes) from the last one:
                           // the previous pass wrote them last, so they are still in L2
+  int nparts;             // inverse x pass: energy partials of the z pass, added by its first CTA
   const float2* tw1;      // fused x/y kernels: W_L1^k, k < L1 (set at launch)
 };
 
@@ -237,6 +238,8 @@ cudaError_t launch_solve_ord(ps_plan_s* p, const T* rho, T* V, double* E, cudaSt
 // energy partials (CTAs of the fused pass) of a plan in another order, and
 // the launch attributes of its kernels
 int ord_conv_ctas(const ps_plan_s* p);
+// CTAs of the z pass (the fused pass) of a plan: its energy partials
+int z_pass_ctas(const ps_plan_s* p);
 template <typename T>
 cudaError_t configure_ord(const ps_plan_s* p);
 // rows of each shared-memory buffer of a generic pass (passes.cu)
@@ -244,7 +247,7 @@ int gen_rows(const ps_plan_s* p, int pass);
 // passes.cu: the generic x pass (P1 forward R2C, P5 inverse C2R) of a plan
 // that processes x first, on A with pitch ld1
 template <typename T>
-cudaError_t launch_x_pass(ps_plan_s* p, int pass, const void* src, void* dst, cudaStream_t s);
+cudaError_t launch_x_pass(ps_plan_s* p, int pass, const void* src, void* dst, double* E, cudaStream_t s);
 cudaError_t build_twiddles(ps_plan_s* p, cudaStream_t s);
 // batch.cu: the batch as one cached CUDA graph of concurrent per-problem chains
 cudaError_t batch_solve_graph(int count, ps_plan_s* const* plans, const void* const* rho, void* const* V,

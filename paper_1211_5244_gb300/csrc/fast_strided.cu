@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q),
       }
     }
     if constexpr (KIND == 2) {
-      if (E != nullptr) energy_finish_f32(eacc, partials, counter, escale, E);
+      if (E != nullptr) energy_partial_f32(eacc, partials);
     }
   }
 }
@@ -376,7 +376,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
     step_tile(nkt, nyi);
   }
   cp_async_wait_all();
-  if (E != nullptr) energy_finish_f32(eacc, partials, counter, escale, E);
+  if (E != nullptr) energy_partial_f32(eacc, partials);
 }
 
 const void* zpipe_u_kernel(int L, bool half, int* threads, size_t* smem, int* tk) {

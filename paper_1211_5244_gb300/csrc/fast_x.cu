@@ -18,6 +18,7 @@
 
 #include "fft_fast.cuh"
 #include "fft_regs.cuh"
+#include "reduce.cuh"
 
 namespace ps {
 
@@ -150,7 +151,7 @@ __global__ void __launch_bounds__(TR*(P < Q ? P : Q), 4)
 template <int P, int Q, int TR, bool HALF, bool SH = false>
 __global__ void __launch_bounds__(TR*(P < Q ? P : Q), SH ? 3 : 4)
     k_x_c2r(const void* src_v, void* dst_v, const float* twm_v, const float2* __restrict__ tw, FastArgs a,
-            double*, unsigned*, double, double*) {
+            double* partials, unsigned*, double escale, double* E) {
   pdl_wait();
   const float2* __restrict__ twm = reinterpret_cast<const float2*>(twm_v);
   using S = XShape<P, Q>;
@@ -249,6 +250,7 @@ __global__ void __launch_bounds__(TR*(P < Q ? P : Q), SH ? 3 : 4)
       }
     }
   }
+  if (E != nullptr && blockIdx.x == 0) energy_total(partials, a.nparts, escale, E);
 }
 
 template <int P, int Q, int TR>
@@ -633,16 +635,17 @@ cudaError_t launch_cfg(const PassCfg& cf, const FastArgs& fa, const void* src, v
 
 }  // namespace
 
-cudaError_t launch_xy(ps_plan_s* p, int kind, const void* src, void* dst, cudaStream_t s) {
+cudaError_t launch_xy(ps_plan_s* p, int kind, const void* src, void* dst, double* E, double escale, cudaStream_t s) {
   const PassCfg& cf = p->xyf[kind];
   FastArgs fa = cf.fa;
+  fa.nparts = z_pass_ctas(p);
   fa.tw1 = static_cast<const float2*>(p->tw[0]);
-  return launch_cfg(cf, fa, src, dst, static_cast<const float*>(p->twx), p->tw4y, nullptr, nullptr, 0.0, nullptr,
+  return launch_cfg(cf, fa, src, dst, static_cast<const float*>(p->twx), p->tw4y, p->partials, nullptr, escale, E,
                     s);
 }
 
-cudaError_t launch_fast_chunk(ps_plan_s* p, int pass, const void* rhoV, void* B, void* A, int z0, int nz,
-                              cudaStream_t s) {
+cudaError_t launch_fast_chunk(ps_plan_s* p, int pass, const void* rhoV, void* B, void* A, int z0, int nz, double* E,
+                              double escale, cudaStream_t s) {
   PassCfg cf = p->cfg[pass];
   FastArgs fa = cf.fa;
   const long long n1 = p->n[0], n2 = p->n[1];
@@ -667,6 +670,7 @@ cudaError_t launch_fast_chunk(ps_plan_s* p, int pass, const void* rhoV, void* B,
       dst = static_cast<float*>(const_cast<void*>(rhoV)) + z0 * n2 * n1;
       break;
   }
+  fa.nparts = z_pass_ctas(p);
   if (pass == P1 || pass == P5) {
     fa.nrows = (int)(nz * n2);
     cf.grid = dim3((unsigned)((fa.nrows + cf.xrows - 1) / cf.xrows));
@@ -678,7 +682,7 @@ cudaError_t launch_fast_chunk(ps_plan_s* p, int pass, const void* rhoV, void* B,
   const float* K = static_cast<const float*>((pass == P1 || pass == P5) ? p->twx : p->K);
   const int axis = pass_axis(p, pass);
   const void* tw = ((pass == P2 && (p->ysoa & 1)) || (pass == P4 && (p->ysoa & 2))) ? p->tw4y : p->tw[axis];
-  return launch_cfg(cf, fa, src, dst, K, tw, p->partials, p->counter, 0.0, nullptr, s);
+  return launch_cfg(cf, fa, src, dst, K, tw, p->partials, p->counter, escale, E, s);
 }
 
 cudaError_t launch_fast(ps_plan_s* p, int pass, const void* src, void* dst, double* E, double escale,
@@ -690,7 +694,9 @@ cudaError_t launch_fast(ps_plan_s* p, int pass, const void* src, void* dst, doub
   const void* tw = (pass == P3 && p->tctab) ? p->tctab
                    : (pass == P3 && p->zsoa_T) ? p->tw4z
                    : ((pass == P2 && (p->ysoa & 1)) || (pass == P4 && (p->ysoa & 2))) ? p->tw4y : p->tw[axis];
-  return launch_cfg(cf, cf.fa, src, dst, K, tw, p->partials, p->counter, escale, E, s);
+  FastArgs fa = cf.fa;
+  fa.nparts = z_pass_ctas(p);
+  return launch_cfg(cf, fa, src, dst, K, tw, p->partials, p->counter, escale, E, s);
 }
 
 }  // namespace ps

@@ -46,6 +46,7 @@
 #include <cooperative_groups.h>
 
 #include "fft_fast.cuh"
+#include "reduce.cuh"
 #include "fft_regs.cuh"
 #include "fft_soa.cuh"
 
@@ -249,7 +250,7 @@ __global__ void __launch_bounds__(kNT, 2)
 template <bool HX>
 __global__ void __launch_bounds__(kNT, 2)
     k_xy_inv(const void* src_v, void* dst_v, const float* twm_v, const float4* __restrict__ tw4, FastArgs a,
-             double*, unsigned*, double, double*) {
+             double* partials, unsigned*, double escale, double* E) {
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank();
   const int z = blockIdx.x / kCS;
@@ -347,6 +348,7 @@ __global__ void __launch_bounds__(kNT, 2)
   float2* vz = reinterpret_cast<float2*>(static_cast<float*>(dst_v) + ((long long)z * a.nrows + row) * a.n1);
 #pragma unroll
   for (int aa = 0; aa < NA; ++aa) vz[j + kXQ * aa] = y[aa];
+  if (E != nullptr && blockIdx.x == 0) energy_total(partials, a.nparts, escale, E);
 }
 
 const void* xy_kernel(int kind, bool half, int* threads, size_t* smem, int* cluster) {

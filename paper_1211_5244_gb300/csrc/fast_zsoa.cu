@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(TK * T, 512 / (TK * T))
     step_tile(nkt, nyi);
   }
   cp_async_wait_all();
-  if (E != nullptr) energy_finish_f32(eacc, partials, counter, escale, E);
+  if (E != nullptr) energy_partial_f32(eacc, partials);
 }
 
 const void* zpipe_kernel(int L, bool half, int* tk_io, int* threads, size_t* smem, int* P_out) {
@@ -498,7 +498,7 @@ __global__ void __launch_bounds__(TK * 8, 4)
     step_tile(nkt, nyi);
   }
   cp_async_wait_all();
-  if (E != nullptr) energy_finish_f32(eacc, partials, counter, escale, E);
+  if (E != nullptr) energy_partial_f32(eacc, partials);
 }
 
 const void* zpipe_q_kernel(int L, bool half, int* threads, size_t* smem, int* tk) {

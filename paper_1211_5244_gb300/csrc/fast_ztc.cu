@@ -423,7 +423,7 @@ __global__ void __launch_bounds__(256, NZ == 8 ? 2 : 1)
   tc::fence_before();
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tb));
-  if (E != nullptr) energy_finish_f32(eacc, partials, counter, escale, E);
+  if (E != nullptr) energy_partial_f32(eacc, partials);
 }
 
 const void* ztc_kernel(int L, bool half, int* threads, size_t* smem) {

@@ -86,14 +86,15 @@ const void* xy_kernel(int kind, bool half, int* threads, size_t* smem, int* clus
 // Fills p->cfg[k].fast / fn / grid / block / smem / fa for the passes covered.
 cudaError_t configure_fast_f32(ps_plan_s* p);
 
-// Launches pass `pass` with its specialised kernel.
+// Launches pass `pass` with its specialised kernel. E (or NULL): the z pass stores
+// its energy partials, the inverse x pass (and the inverse fused x/y kernel) adds them.
 cudaError_t launch_fast(ps_plan_s* p, int pass, const void* src, void* dst, double* E, double escale,
                         cudaStream_t s);
 // Launches the fused forward (kind 0: rho -> B) or inverse (kind 1: B -> V) x/y kernel.
-cudaError_t launch_xy(ps_plan_s* p, int kind, const void* src, void* dst, cudaStream_t s);
+cudaError_t launch_xy(ps_plan_s* p, int kind, const void* src, void* dst, double* E, double escale, cudaStream_t s);
 // Launches x pass P1 / P5 or y pass P2 / P4 on the z planes z0 .. z0 + nz - 1:
 // rho, V and B at those planes, A (src or dst) at its first plane.
 cudaError_t launch_fast_chunk(ps_plan_s* p, int pass, const void* rhoV, void* B, void* A, int z0, int nz,
-                              cudaStream_t s);
+                              double* E, double escale, cudaStream_t s);
 
 }  // namespace ps

@@ -180,8 +180,7 @@ __global__ void __launch_bounds__(256) py_generic(const cpx<T>* __restrict__ src
 template <typename T, int BM = 0>
 __global__ void __launch_bounds__(256) pz_generic(cpx<T>* __restrict__ Bw, const T* __restrict__ K,
                                                   const cpx<T>* __restrict__ tw, GenArgs a,
-                                                  double* partials, unsigned* counter,
-                                                  double escale, double* E) {
+                                                  double* partials, double* E) {
   using C = cpx<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf0 = reinterpret_cast<C*>(smem_raw);
@@ -244,14 +243,15 @@ __global__ void __launch_bounds__(256) pz_generic(cpx<T>* __restrict__ Bw, const
     const int t = w & (a.tk - 1), z = w >> a.ltk;
     if (kx0 + t < a.c) line[z * zstride + t] = res[z * a.ldt + t];
   }
-  if (E != nullptr) energy_finish((double)eacc, partials, counter, escale, E);
+  if (E != nullptr) energy_partial((double)eacc, partials);
 }
 
 // ---------------------------------------------------------------- P5
 
 template <typename T, int BM = 0>
 __global__ void __launch_bounds__(256) p5_generic(const cpx<T>* __restrict__ A, T* __restrict__ V,
-                                                  const cpx<T>* __restrict__ tw, GenArgs a) {
+                                                  const cpx<T>* __restrict__ tw, GenArgs a, const double* partials,
+                                                  int nparts, double escale, double* E) {
   using C = cpx<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf0 = reinterpret_cast<C*>(smem_raw);
@@ -332,6 +332,7 @@ __global__ void __launch_bounds__(256) p5_generic(const cpx<T>* __restrict__ A, 
     }
     V[(size_t)row * a.n1 + i] = v;
   }
+  if (E != nullptr && blockIdx.x == 0) energy_total(partials, nparts, escale, E);
 }
 
 // ---------------------------------------------------------------- kernel table
@@ -344,8 +345,8 @@ struct GenKernels {
   void (*p1)(const T*, cpx<T>*, const cpx<T>*, GenArgs);
   void (*pyf)(const cpx<T>*, cpx<T>*, const cpx<T>*, GenArgs);
   void (*pyi)(const cpx<T>*, cpx<T>*, const cpx<T>*, GenArgs);
-  void (*pz)(cpx<T>*, const T*, const cpx<T>*, GenArgs, double*, unsigned*, double, double*);
-  void (*p5)(const cpx<T>*, T*, const cpx<T>*, GenArgs);
+  void (*pz)(cpx<T>*, const T*, const cpx<T>*, GenArgs, double*, double*);
+  void (*p5)(const cpx<T>*, T*, const cpx<T>*, GenArgs, const double*, int, double, double*);
 };
 
 template <typename T, int BM>
@@ -495,6 +496,13 @@ int gen_rows(const ps_plan_s* p, int pass) {
   return r;
 }
 
+int z_pass_ctas(const ps_plan_s* p) {
+  if (p->cfg[P3].fast && (canonical_order(p) || p->fastord)) return (int)(p->cfg[P3].grid.x * p->cfg[P3].grid.y);
+  if (p->tile[P3].on) return (int)(p->tile[P3].grid.x * p->tile[P3].grid.y);
+  if (!canonical_order(p)) return ord_conv_ctas(p);
+  return (p->c + p->cfg[P3].tk - 1) / p->cfg[P3].tk * p->L[1];
+}
+
 template <typename T>
 static GenArgs gen_args(const ps_plan_s* p, int pass) {
   GenArgs a;
@@ -640,7 +648,7 @@ cudaError_t launch_solve(ps_plan_s* p, const T* rho, T* V, double* E, cudaStream
     GenArgs a = gen_args<T>(p, P3);
     dim3 g((p->c + a.tk - 1) / a.tk, p->L[1]);
     gen_kernels<T>(p->cfg[P3].bm).pz<<<g, p->cfg[P3].threads, p->cfg[P3].gsmem, s>>>(
-        B, static_cast<const T*>(p->K), tw2, a, p->partials, p->counter, escale, E);
+        B, static_cast<const T*>(p->K), tw2, a, p->partials, E);
     return cudaGetLastError();
   };
   if (!xyf && a8 && p->chunks > 1) {
@@ -650,8 +658,8 @@ cudaError_t launch_solve(ps_plan_s* p, const T* rho, T* V, double* E, cudaStream
     if (ev) cudaEventRecord(ev[0], s);
     for (int z0 = 0; z0 < n3; z0 += nz) {
       const int cz = std::min(nz, n3 - z0);
-      if ((e = launch_fast_chunk(p, P1, rho, B, A, z0, cz, s)) != cudaSuccess) return e;
-      if ((e = launch_fast_chunk(p, P2, rho, B, A, z0, cz, s)) != cudaSuccess) return e;
+      if ((e = launch_fast_chunk(p, P1, rho, B, A, z0, cz, nullptr, 0.0, s)) != cudaSuccess) return e;
+      if ((e = launch_fast_chunk(p, P2, rho, B, A, z0, cz, nullptr, 0.0, s)) != cudaSuccess) return e;
     }
     if (ev) cudaEventRecord(ev[1], s);
     if (ev) cudaEventRecord(ev[2], s);
@@ -659,8 +667,8 @@ cudaError_t launch_solve(ps_plan_s* p, const T* rho, T* V, double* E, cudaStream
     if (ev) cudaEventRecord(ev[3], s);
     for (int z0 = 0; z0 < n3; z0 += nz) {
       const int cz = std::min(nz, n3 - z0);
-      if ((e = launch_fast_chunk(p, P4, V, B, A, z0, cz, s)) != cudaSuccess) return e;
-      if ((e = launch_fast_chunk(p, P5, V, B, A, z0, cz, s)) != cudaSuccess) return e;
+      if ((e = launch_fast_chunk(p, P4, V, B, A, z0, cz, nullptr, 0.0, s)) != cudaSuccess) return e;
+      if ((e = launch_fast_chunk(p, P5, V, B, A, z0, cz, z0 == 0 ? Ez : nullptr, escale, s)) != cudaSuccess) return e;
     }
     if ((e = energy_after()) != cudaSuccess) return e;
     if (ev) cudaEventRecord(ev[4], s);
@@ -670,7 +678,7 @@ cudaError_t launch_solve(ps_plan_s* p, const T* rho, T* V, double* E, cudaStream
   if (ev) cudaEventRecord(ev[0], s);
   // P1
   if (xyf) {
-    if ((e = launch_xy(p, 0, rho, B, s)) != cudaSuccess) return e;
+    if ((e = launch_xy(p, 0, rho, B, nullptr, 0.0, s)) != cudaSuccess) return e;
   } else if (p->cfg[P1].fast && a8) {
     if ((e = launch_fast(p, P1, rho, A, nullptr, 0.0, s)) != cudaSuccess) return e;
   } else if (p->tile[P1].on) {
@@ -700,7 +708,7 @@ cudaError_t launch_solve(ps_plan_s* p, const T* rho, T* V, double* E, cudaStream
   if (ev) cudaEventRecord(ev[3], s);
   // P4
   if (xyf) {
-    if ((e = launch_xy(p, 1, B, V, s)) != cudaSuccess) return e;
+    if ((e = launch_xy(p, 1, B, V, Ez, escale, s)) != cudaSuccess) return e;
   } else if (p->cfg[P4].fast) {
     if ((e = launch_fast(p, P4, B, A, nullptr, 0.0, s)) != cudaSuccess) return e;
   } else if (p->tile[P4].on) {
@@ -715,14 +723,14 @@ cudaError_t launch_solve(ps_plan_s* p, const T* rho, T* V, double* E, cudaStream
   if (xyf) {
     // done by the fused kernel above
   } else if (p->cfg[P5].fast && a8) {
-    if ((e = launch_fast(p, P5, A, V, nullptr, 0.0, s)) != cudaSuccess) return e;
+    if ((e = launch_fast(p, P5, A, V, Ez, escale, s)) != cudaSuccess) return e;
   } else if (p->tile[P5].on) {
-    if ((e = launch_tile(p, P5, A, V, nullptr, s)) != cudaSuccess) return e;
+    if ((e = launch_tile(p, P5, A, V, Ez, s)) != cudaSuccess) return e;
   } else {
     GenArgs a = gen_args<T>(p, P5);
     const int rpc = (p->L[0] % 2 == 0) ? a.tk : 2 * a.tk;  // odd L1: two real rows per line
     gen_kernels<T>(p->cfg[P5].bm).p5<<<(nrows + rpc - 1) / rpc, p->cfg[P5].threads, p->cfg[P5].gsmem, s>>>(
-        A, V, tw0, a);
+        A, V, tw0, a, p->partials, z_pass_ctas(p), escale, Ez);
   }
   if ((e = energy_after()) != cudaSuccess) return e;
   if (ev) cudaEventRecord(ev[5], s);
@@ -730,7 +738,7 @@ cudaError_t launch_solve(ps_plan_s* p, const T* rho, T* V, double* E, cudaStream
 }
 
 template <typename T>
-cudaError_t launch_x_pass(ps_plan_s* p, int pass, const void* src, void* dst, cudaStream_t s) {
+cudaError_t launch_x_pass(ps_plan_s* p, int pass, const void* src, void* dst, double* E, cudaStream_t s) {
   using C = cpx<T>;
   GenArgs a = gen_args<T>(p, pass);
   const int nrows = p->n[1] * p->n[2];
@@ -741,12 +749,13 @@ cudaError_t launch_x_pass(ps_plan_s* p, int pass, const void* src, void* dst, cu
         static_cast<const T*>(src), static_cast<C*>(dst), tw0, a);
   else
     gen_kernels<T>(p->cfg[P5].bm).p5<<<(nrows + rpc - 1) / rpc, p->cfg[P5].threads, p->cfg[P5].gsmem, s>>>(
-        static_cast<const C*>(src), static_cast<T*>(dst), tw0, a);
+        static_cast<const C*>(src), static_cast<T*>(dst), tw0, a, p->partials, z_pass_ctas(p),
+        0.5 * p->h * p->h * p->h, E);
   return cudaGetLastError();
 }
 
-template cudaError_t launch_x_pass<float>(ps_plan_s*, int, const void*, void*, cudaStream_t);
-template cudaError_t launch_x_pass<double>(ps_plan_s*, int, const void*, void*, cudaStream_t);
+template cudaError_t launch_x_pass<float>(ps_plan_s*, int, const void*, void*, double*, cudaStream_t);
+template cudaError_t launch_x_pass<double>(ps_plan_s*, int, const void*, void*, double*, cudaStream_t);
 template cudaError_t configure_passes<float>(ps_plan_s*);
 template cudaError_t configure_passes<double>(ps_plan_s*);
 template cudaError_t launch_solve<float>(ps_plan_s*, const float*, float*, double*, cudaStream_t,

@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(256) ord_line(const cpx<T>* __restrict__ src, 
 template <typename T>
 __global__ void __launch_bounds__(256) ord_conv(cpx<T>* __restrict__ X, const T* __restrict__ K,
                                                 const cpx<T>* __restrict__ tw, OrdArgs a, double* partials,
-                                                unsigned* counter, double escale, double* E) {
+                                                double* E) {
   using C = cpx<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf0 = reinterpret_cast<C*>(smem_raw);
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(256) ord_conv(cpx<T>* __restrict__ X, const T*
   __syncthreads();
   C* res = line_transform<1, T>(spec, other, a.N, a.tk, a.ldt, a.st, ttab, tstr, a.bl);
   store_tile<T>(line, res, a, t0);
-  if (E != nullptr) energy_finish((double)eacc, partials, counter, escale, E);
+  if (E != nullptr) energy_partial((double)eacc, partials);
 }
 
 // P1 along y or z: real columns x = 2 (t0 + t) and x + 1 as one complex line
@@ -187,7 +187,8 @@ __global__ void __launch_bounds__(256) ord_r2c(const T* __restrict__ rho, cpx<T>
 // P5 along y or z: the inverse of ord_r2c
 template <typename T>
 __global__ void __launch_bounds__(256) ord_c2r(const cpx<T>* __restrict__ A, T* __restrict__ V,
-                                               const cpx<T>* __restrict__ tw, OrdArgs a) {
+                                               const cpx<T>* __restrict__ tw, OrdArgs a, const double* partials,
+                                               int nparts, double escale, double* E) {
   using C = cpx<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf0 = reinterpret_cast<C*>(smem_raw);
@@ -229,6 +230,7 @@ __global__ void __launch_bounds__(256) ord_c2r(const cpx<T>* __restrict__ A, T* 
     const C v = z[e * a.ldt + (xl >> 1)];
     dst[(long long)e * a.se_out + xl] = (xl & 1) ? v.y : v.x;
   }
+  if (E != nullptr && blockIdx.x == 0 && blockIdx.y == 0) energy_total(partials, nparts, escale, E);
 }
 
 // strides (x, y, z) of an x-fastest array with extents e and x pitch ld
@@ -355,7 +357,7 @@ cudaError_t launch_solve_ord(ps_plan_s* p, const T* rho, T* V, double* E, cudaSt
   if (p->tile[P1].on) {
     if ((e = launch_tile(p, P1, rho, A, nullptr, s)) != cudaSuccess) return e;
   } else if (xfirst) {
-    if ((e = launch_x_pass<T>(p, P1, rho, A, s)) != cudaSuccess) return e;
+    if ((e = launch_x_pass<T>(p, P1, rho, A, nullptr, s)) != cudaSuccess) return e;
   } else {
     OrdArgs a = ord_args<T>(p, P1, &g);
     ord_r2c<T><<<g, p->cfg[P1].threads, p->cfg[P1].gsmem, s>>>(rho, A, tw(P1), a);
@@ -373,8 +375,7 @@ cudaError_t launch_solve_ord(ps_plan_s* p, const T* rho, T* V, double* E, cudaSt
   } else {
     OrdArgs a = ord_args<T>(p, P3, &g);
     ord_conv<T><<<g, p->cfg[P3].threads, p->cfg[P3].gsmem, s>>>(B, static_cast<const T*>(p->K), tw(P3), a,
-                                                                p->partials, p->counter,
-                                                                0.5 * p->h * p->h * p->h, E);
+                                                                p->partials, E);
   }
   if (ev) cudaEventRecord(ev[3], s);
   if (p->tile[P4].on) {
@@ -385,12 +386,13 @@ cudaError_t launch_solve_ord(ps_plan_s* p, const T* rho, T* V, double* E, cudaSt
   }
   if (ev) cudaEventRecord(ev[4], s);
   if (p->tile[P5].on) {
-    if ((e = launch_tile(p, P5, A, V, nullptr, s)) != cudaSuccess) return e;
+    if ((e = launch_tile(p, P5, A, V, E, s)) != cudaSuccess) return e;
   } else if (xfirst) {
-    if ((e = launch_x_pass<T>(p, P5, A, V, s)) != cudaSuccess) return e;
+    if ((e = launch_x_pass<T>(p, P5, A, V, E, s)) != cudaSuccess) return e;
   } else {
     OrdArgs a = ord_args<T>(p, P5, &g);
-    ord_c2r<T><<<g, p->cfg[P5].threads, p->cfg[P5].gsmem, s>>>(A, V, tw(P5), a);
+    ord_c2r<T><<<g, p->cfg[P5].threads, p->cfg[P5].gsmem, s>>>(A, V, tw(P5), a, p->partials, z_pass_ctas(p),
+                                                               0.5 * p->h * p->h * p->h, E);
   }
   if (ev) cudaEventRecord(ev[5], s);
   return cudaGetLastError();

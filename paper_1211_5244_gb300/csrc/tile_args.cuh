@@ -38,8 +38,9 @@ struct TileArgs {
   // La0 / 2
   int Lt, Lp, La0, w_tile;
   int Kst, Ksp, Kse;
+  // energy: partials of the fused pass, added by the last pass's first CTA
   double* partials;
-  unsigned* counter;
+  int nparts;
   double escale;
   double* E;
   // real passes: line t holds two real sequences (or the even and odd elements

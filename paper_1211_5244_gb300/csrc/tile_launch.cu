@@ -310,9 +310,9 @@ cudaError_t launch_tile(ps_plan_s* p, int pass, const void* src, void* dst, doub
   a.K = p->K;
   a.tw = a.twL = p->tw[al];
   a.partials = p->partials;
-  a.counter = p->counter;
+  a.nparts = z_pass_ctas(p);
   a.escale = 0.5 * p->h * p->h * p->h;
-  a.E = pass == P3 ? E : nullptr;
+  a.E = E;
   if (a.vec) {
     const void* r = pass == P1 ? src : dst;
     a.vec = reinterpret_cast<uintptr_t>(r) % (2 * p->esz) == 0;

@@ -23,6 +23,7 @@
 #pragma once
 
 #include "fft_fast.cuh"
+#include "reduce.cuh"
 #include "tile_dft.cuh"
 
 namespace ps {
@@ -303,44 +304,6 @@ __global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_line(const
 
 // ------------------------------------------------------------ forward, K^F, inverse
 
-// The energy of the fused pass, in two halves around the inverse transform so
-// that its fence and atomic run beside it instead of holding every CTA at its end
-// (L = 220, 18180 lines on 2273 CTAs: 47.3 us with the reduction at the end).
-// Before a barrier: the warp sums. After it: energy_arrive in thread 0 adds
-// them, stores the CTA's partial and counts its arrival. At the end the first warp of
-// the CTA that arrived last adds all partials in index order and resets the counter.
-template <typename T>
-__device__ __forceinline__ void energy_warps(T en, T* wsum) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) en += __shfl_xor_sync(0xffffffffu, en, o);
-  if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = en;
-}
-template <typename T>
-__device__ __forceinline__ unsigned energy_arrive(const TileArgs& a, const T* wsum) {
-  double sum = 0.0;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) sum += (double)wsum[w];
-  a.partials[blockIdx.y * gridDim.x + blockIdx.x] = sum;
-  __threadfence();
-  return atomicAdd(a.counter, 1u);
-}
-__device__ __forceinline__ void energy_last(const TileArgs& a, unsigned arrived) {
-  const unsigned n = gridDim.x * gridDim.y;
-  if (__shfl_sync(0xffffffffu, arrived, 0) != n - 1) return;
-  __threadfence();
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  for (unsigned i = threadIdx.x; i < n; i += 128)
-#pragma unroll
-    for (unsigned u = 0; u < 4; ++u)
-      if (i + 32 * u < n) acc[u] += __ldcg(a.partials + i + 32 * u);
-  double sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-  if (threadIdx.x == 0) {
-    *a.E = a.escale * sum;
-    *a.counter = 0u;
-  }
-}
-
 template <typename T, bool HALF, int CLS>
 __global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_conv(const __grid_constant__ TileArgs a) {
   using C = cpx<T>;
@@ -399,10 +362,17 @@ __global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_conv(const
       for (int r = 0; r < R; ++r) p[r * a.es] = x[r];
     });
   });
-  if (a.E != nullptr) energy_warps(en, wsum);
+  if (a.E != nullptr) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) en += __shfl_xor_sync(0xffffffffu, en, o);
+    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = en;
+  }
   __syncthreads();
-  unsigned arrived = 0;
-  if (a.E != nullptr && threadIdx.x == 0) arrived = energy_arrive(a, wsum);
+  if (a.E != nullptr && threadIdx.x == 0) {  // the CTA's partial (energy_total adds them in the last pass)
+    double sum = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) sum += (double)wsum[w];
+    a.partials[blockIdx.y * gridDim.x + blockIdx.x] = sum;
+  }
   step_middle<1, CLS>(a, s);
   step_final<HALF, CLS>(a, s, [&](int t) {
     bool ok;
@@ -411,7 +381,6 @@ __global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_conv(const
       if (ok && e < a.nout) dst[(long long)e * a.se_out] = v;
     };
   });
-  if (a.E != nullptr && threadIdx.x < 32) energy_last(a, arrived);
 }
 
 // ------------------------------------------------------------ real passes
@@ -526,6 +495,7 @@ __global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_c2r(const 
       }
     };
   });
+  if (a.E != nullptr && blockIdx.x == 0 && blockIdx.y == 0) energy_total(a.partials, a.nparts, a.escale, a.E);
 }
 
 }  // namespace tile
