@@ -15,19 +15,14 @@
 // kernel: the inverse's first step needs exactly the k1 values the forward's
 // last step left in each thread, so the spectrum never leaves registers.
 #include "fft_fast.cuh"
-#include "fft_regs.cuh"
 #include "reduce.cuh"
+#include "tile_dft.cuh"
 
 namespace ps {
 
-using regs::rdft;
-
-__device__ __forceinline__ float2 cmulf(float2 a, float2 b) {
-  return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-__device__ __forceinline__ float2 cmulcf(float2 a, float2 b) {
-  return make_float2(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
-}
+using tile::dft;
+using tile::dft_pre;
+using tile::full_mask;
 
 constexpr int kTK = 16;  // lines per CTA
 
@@ -72,9 +67,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q),
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
       const int b = j + T * u;
-      rdft<P, -1, HALF>(y[u]);
-#pragma unroll
-      for (int k1 = 1; k1 < P; ++k1) y[u][k1] = cmulf(y[u][k1], __ldg(&tw[b * k1]));
+      dft<P, -1, full_mask(NA)>(y[u]);
 #pragma unroll
       for (int k1 = 0; k1 < P; ++k1) sh[(b * P + k1) * TK + t] = y[u][k1];
     }
@@ -84,7 +77,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q),
       const int k1 = j + T * v;
 #pragma unroll
       for (int b = 0; b < Q; ++b) X[v][b] = sh[(b * P + k1) * TK + t];
-      rdft<Q, -1, false>(X[v]);
+      dft_pre<Q, -1>(X[v], tw, k1, P);
     }
   } else {
 #pragma unroll
@@ -128,14 +121,11 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q),
       }
       eacc *= (kx == 0 || 2 * kx == a.L1) ? 1.f : 2.f;
     }
-    // inverse: Q-point transforms over k2, conjugate twiddles, exchange,
+    // inverse: Q-point transforms over k2, exchange, conjugate twiddles and
     // P-point transforms over k1
 #pragma unroll
     for (int v = 0; v < NK; ++v) {
-      const int k1 = j + T * v;
-      rdft<Q, 1, false>(X[v]);
-#pragma unroll
-      for (int b = 1; b < Q; ++b) X[v][b] = cmulcf(X[v][b], __ldg(&tw[b * k1]));
+      dft<Q, 1, full_mask(Q)>(X[v]);
     }
     if constexpr (KIND == 2) __syncthreads();  // the forward exchange has been read
 #pragma unroll
@@ -151,7 +141,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q),
       float2 y[P];
 #pragma unroll
       for (int k1 = 0; k1 < P; ++k1) y[k1] = sh[(b * P + k1) * TK + t];
-      rdft<P, 1, false>(y);
+      dft_pre<P, 1>(y, tw, b, Q);
       if (valid) {
 #pragma unroll
         for (int aa = 0; aa < NA; ++aa)
@@ -312,9 +302,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
       const int b = j + T * u;
-      rdft<P, -1, HALF>(y[u]);
-#pragma unroll
-      for (int k1 = 1; k1 < P; ++k1) y[u][k1] = cmulf(y[u][k1], tws[b * k1]);
+      dft<P, -1, full_mask(NA)>(y[u]);
 #pragma unroll
       for (int k1 = 0; k1 < P; ++k1) sh[(b * PP + k1) * TK + t] = y[u][k1];
     }
@@ -326,7 +314,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
       const int k1 = j + T * v;
 #pragma unroll
       for (int b = 0; b < Q; ++b) X[v][b] = sh[(b * PP + k1) * TK + t];
-      rdft<Q, -1, false>(X[v]);
+      dft_pre<Q, -1>(X[v], tws, k1, P);
       // V^F = K^F rho^F on the even octant of K^F; energy sum K |rho^F|^2
 #pragma unroll
       for (int k2 = 0; k2 < Q; ++k2) {
@@ -337,9 +325,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
         e1 = fmaf(kk, x.x * x.x + x.y * x.y, e1);
         X[v][k2] = make_float2(kk * x.x, kk * x.y);
       }
-      rdft<Q, 1, false>(X[v]);
-#pragma unroll
-      for (int b = 1; b < Q; ++b) X[v][b] = cmulcf(X[v][b], tws[b * k1]);
+      dft<Q, 1, full_mask(Q)>(X[v]);
     }
     eacc += e1 * ((kx == 0 || 2 * kx == a.L1) ? 1.f : 2.f);
     __syncthreads();  // the forward exchange and the K^F slice have been read
@@ -364,7 +350,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
       const int b = j + T * u;
-      rdft<P, 1, false>(y[u]);
+      dft_pre<P, 1>(y[u], tws, b, Q);
       if (valid) {
 #pragma unroll
         for (int aa = 0; aa < NA; ++aa)
@@ -503,9 +489,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
 #pragma unroll
       for (int u = 0; u < NB; ++u) {
         const int b = j + T * u;
-        rdft<P, -1, HALF>(y[u]);
-#pragma unroll
-        for (int k1 = 1; k1 < P; ++k1) y[u][k1] = cmulf(y[u][k1], __ldg(&tw[b * k1]));
+        dft<P, -1, full_mask(NA)>(y[u]);
 #pragma unroll
         for (int k1 = 0; k1 < P; ++k1) sh[(b * PP + k1) * TK + t] = y[u][k1];
       }
@@ -522,7 +506,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
 #pragma unroll
       for (int v = 0; v < NK; ++v) {
         const int k1 = j + T * v;
-        rdft<Q, -1, false>(X[v]);
+        dft_pre<Q, -1>(X[v], tw, k1, P);
         if (valid) {
 #pragma unroll
           for (int k2 = 0; k2 < Q; ++k2) d[(long long)(k1 + P * k2) * a.dst_elem] = X[v][k2];
@@ -540,9 +524,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
 #pragma unroll
       for (int v = 0; v < NK; ++v) {
         const int k1 = j + T * v;
-        rdft<Q, 1, false>(X[v]);
-#pragma unroll
-        for (int b = 1; b < Q; ++b) X[v][b] = cmulcf(X[v][b], __ldg(&tw[b * k1]));
+        dft<Q, 1, full_mask(Q)>(X[v]);
 #pragma unroll
         for (int b = 0; b < Q; ++b) sh[(b * PP + k1) * TK + t] = X[v][b];
       }
@@ -560,7 +542,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
 #pragma unroll
       for (int u = 0; u < NB; ++u) {
         const int b = j + T * u;
-        rdft<P, 1, false>(y[u]);
+        dft_pre<P, 1>(y[u], tw, b, Q);
         if (valid) {
 #pragma unroll
           for (int aa = 0; aa < NA; ++aa)
