@@ -41,6 +41,7 @@ struct TileArgs {
   // energy: partials of the fused pass, added by the last pass's first CTA
   double* partials;
   int nparts;
+  int shift;  // 1: the first CTA in x adds the partials and has no lines
   double escale;
   double* E;
   // real passes: line t holds two real sequences (or the even and odd elements

@@ -320,6 +320,10 @@ cudaError_t launch_tile(ps_plan_s* p, int pass, const void* src, void* dst, doub
   void* args[] = {(void*)&a};
   cudaLaunchConfig_t lc = {};
   lc.gridDim = tl.grid;
+  if (pass == P5 && E != nullptr) {
+    a.shift = 1;
+    ++lc.gridDim.x;
+  }
   lc.blockDim = dim3((unsigned)tl.threads);
   lc.dynamicSmemBytes = tl.smem;
   lc.stream = s;
