@@ -156,6 +156,42 @@ int bluestein_length(int N, int max_M) {
   return best ? best : first;
 }
 
+// Bluestein for transform lengths with a prime factor >= 11 (a direct sum
+// over that factor would cost N * p per line), if M fits the tile. `stockham`: for
+// the kernels of passes.cu, else for the tile kernels where they have a length.
+void choose_bluestein(ps_plan_s* p, int j, bool stockham) {
+  const int N = xform_len(p, j);
+  int big = 1;
+  for (int r = 0; r < p->st[j].n; ++r) big = p->st[j].R[r] > big ? p->st[j].R[r] : big;
+  p->blue[j] = BlueArgs{};
+  TileRadix tr;
+  if (big < 11 || (!stockham && tile_radix(N, N % 2 == 0, p->dtype == PS_F32, &tr))) return;
+  // two buffers of M rows for a one-line tile (ldt = 2) must fit the
+  // 200 KiB shared-memory budget of the generic kernels
+  const size_t csz = 2 * (p->dtype == PS_F32 ? 4 : 8);
+  const int max_M = (int)std::min<size_t>(kMaxLen, 200 * 1024 / (2 * 2 * csz));
+  int M = bluestein_length(N, max_M);
+  // FP32: the shortest length >= 2N where the register four-step form
+  // exists (a power of two or 3 * 2^k up to 384: up to twice the points of
+  // the smooth length, at a fraction of the cost per point of the
+  // Stockham stages); PS_BLUE_REGS=0 (or PS_BLUE_M=min) keeps the smooth length
+  const char* rv = getenv("PS_BLUE_REGS");
+  const char* mv = getenv("PS_BLUE_M");
+  const bool regs = !(rv && atoi(rv) == 0) && !(mv && strcmp(mv, "min") == 0);
+  int m2 = 0;
+  for (const int v : {32, 64, 96, 128, 192, 256, 384})
+    if (m2 == 0 && v >= 2 * N) m2 = v;
+  if (p->dtype == PS_F32 && regs && m2 && blue_regs_length(m2, N)) M = m2;
+  if (regs && !stockham) {
+    const int mt = tile_blue_length(N, p->dtype == PS_F32, max_M);
+    if (mt) M = mt;
+  }
+  if (M <= max_M) {
+    p->blue[j].M = M;
+    p->blue[j].st = factorize(M);
+  }
+}
+
 int check_solve_args(ps_plan p, const void* in, const void* out) {
   if (!p) return fail(PS_ERR_ARG, "plan is NULL");
   if (!in || !out) return fail(PS_ERR_ARG, "input or output pointer is NULL");
@@ -255,36 +291,7 @@ int ps_plan_set_lengths(ps_plan p, int L1, int L2, int L3) {
   const int a0 = p->ord[0], a1 = p->ord[1];
   p->c = p->L[a0] / 2 + 1;  // outputs kept by the real-to-complex transform (§3)
   for (int j = 0; j < 3; ++j) p->st[j] = factorize(xform_len(p, j));
-  // Bluestein for transform lengths with a prime factor >= 11 (a direct sum
-  // over that factor would cost N * p per line), if M fits the tile
-  for (int j = 0; j < 3; ++j) {
-    const int N = xform_len(p, j);
-    int big = 1;
-    for (int r = 0; r < p->st[j].n; ++r) big = p->st[j].R[r] > big ? p->st[j].R[r] : big;
-    p->blue[j] = BlueArgs{};
-    if (big >= 11) {
-      // two buffers of M rows for a one-line tile (ldt = 2) must fit the
-      // 200 KiB shared-memory budget of the generic kernels
-      const size_t csz = 2 * (p->dtype == PS_F32 ? 4 : 8);
-      const int max_M = (int)std::min<size_t>(kMaxLen, 200 * 1024 / (2 * 2 * csz));
-      int M = bluestein_length(N, max_M);
-      // FP32: the shortest length >= 2N where the register four-step form
-      // exists (a power of two or 3 * 2^k up to 384: up to twice the points of
-      // the smooth length, at a fraction of the cost per point of the
-      // Stockham stages); PS_BLUE_REGS=0 (or PS_BLUE_M=min) keeps the smooth length
-      const char* rv = getenv("PS_BLUE_REGS");
-      const char* mv = getenv("PS_BLUE_M");
-      const bool regs = !(rv && atoi(rv) == 0) && !(mv && strcmp(mv, "min") == 0);
-      int m2 = 0;
-      for (const int v : {32, 64, 96, 128, 192, 256, 384})
-        if (m2 == 0 && v >= 2 * N) m2 = v;
-      if (p->dtype == PS_F32 && regs && m2 && blue_regs_length(m2, N)) M = m2;
-      if (M <= max_M) {
-        p->blue[j].M = M;
-        p->blue[j].st = factorize(M);
-      }
-    }
-  }
+  for (int j = 0; j < 3; ++j) choose_bluestein(p, j, false);
   // the arrays after the first forward pass (extent c along the first axis)
   // and after the second (the second axis at its padded length), x fastest
   // with a pitch of 128 bytes
@@ -436,6 +443,8 @@ int ps_kernel_build(ps_plan p, void* stream) {
   for (int j = 0; j < 3; ++j) {  // the schedule's radix split of the generic stages, per axis
     const int r = axis_radix(p, j);
     if (!r) continue;
+    p->st[j] = factorize(xform_len(p, j));
+    choose_bluestein(p, j, true);
     p->st[j] = factorize(xform_len(p, j), r);
     if (p->blue[j].M) p->blue[j].st = factorize(p->blue[j].M, r);
   }

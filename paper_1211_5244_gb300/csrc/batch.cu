@@ -76,7 +76,7 @@ double solve_cost(const ps_plan_s* p) {
   auto f = [&](int j, int N) -> double {
     if (N < 2) return 0.0;
     bool tiled = false;  // the tile kernels need no convolution
-    for (int k = 0; k < 5; ++k) tiled |= pass_axis(p, k) == j && p->tile[k].on;
+    for (int k = 0; k < 5; ++k) tiled |= pass_axis(p, k) == j && p->tile[k].on && !p->tile[k].blue;
     const int M = tiled ? 0 : p->blue[j].M;
     return M ? 2.0 * M * std::log2((double)M) + 3.0 * N : N * std::log2((double)N);
   };

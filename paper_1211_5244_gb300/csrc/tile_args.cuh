@@ -53,10 +53,15 @@ struct TileArgs {
   int nreal;   // reals of a row (even x passes), or real sequences in all (pairs)
   int vec;     // real pairs are adjacent and aligned: one access each
   unsigned mout;  // div_magic of the outputs per line in the untangling loop
+  // Bluestein form: N is the convolution length, Nt the line's; the chirp and its transform
+  int Nt;
+  const void* chirp;
+  const void* Bf;
 };
 
 struct TileLaunch {
   int on;           // the pass runs on the tile kernels
+  int blue;         // in Bluestein form
   const void* fn;
   dim3 grid;
   int threads;
@@ -66,13 +71,18 @@ struct TileLaunch {
 
 // Factorisation of N into two (or three) register steps; false if there is none.
 struct TileRadix { int Ra, Rm, Rl, cls; };
-bool tile_radix(int N, bool even_first, bool f32, TileRadix* r);
+bool tile_radix(int N, bool even_first, bool f32, TileRadix* r, double* cost = nullptr);
+// Convolution length of the Bluestein form of a length-N transform on the tile
+// kernels, at most max_M (0: none).
+int tile_blue_length(int N, bool f32, int max_M);
 
 // kernels by kind (tile_*.cu): cls 0 radices up to 8, 1 up to 16; half: n <= N / 2
 template <typename T> const void* tile_line_kernel(int dir, bool half, int cls);
 template <typename T> const void* tile_conv_kernel(bool half, int cls);
 template <typename T> const void* tile_r2c_kernel(bool pair, bool half, int cls);
 template <typename T> const void* tile_c2r_kernel(bool pair, bool half, int cls);
+// the same passes in Bluestein form: P1 .. P5
+template <typename T> const void* tile_blue_kernel(int pass, bool pair);
 
 // Fills p->tile[pass] for the passes that run here (before npart is taken).
 template <typename T> cudaError_t configure_tile(ps_plan_s* p);

@@ -46,7 +46,7 @@ double dft_pre_ops(int R) {
 // A length with one prime factor from 17 to 31 takes it as its last radix: about p + 3
 // operations per element, where the Bluestein convolution of passes.cu runs two
 // transforms of at least twice the length.
-bool tile_radix(int N, bool even_first, bool f32, TileRadix* out) {
+bool tile_radix(int N, bool even_first, bool f32, TileRadix* out, double* cost) {
   constexpr int kMax = 16;
   const double step = f32 ? 2.0 : 0.0;
   auto small = [](int R) { return R == 2 ? 4.0 : 0.0; };
@@ -58,6 +58,7 @@ bool tile_radix(int N, bool even_first, bool f32, TileRadix* out) {
     if (best < 0.0 || c < best) {
       best = c;
       *out = TileRadix{Ra, Rm, Rl, cls};
+      if (cost) *cost = c;
     }
   };
   for (int Ra = 2; Ra <= kMax; ++Ra) {
@@ -74,6 +75,23 @@ bool tile_radix(int N, bool even_first, bool f32, TileRadix* out) {
       if (q % Ra == 0 && q / Ra <= kMax && !(even_first && Ra % 2)) consider(Ra, q / Ra, p, 2);
   }
   return best >= 0.0;
+}
+
+// The even M from 2 N (half of the convolution's input is zero) to 4 N with the
+// least operations per line: its two transforms and the product with Bf.
+int tile_blue_length(int N, bool f32, int max_M) {
+  int best_M = 0;
+  double best = 0.0;
+  for (int M = 2 * N; M <= 4 * N && M <= max_M; M += 2) {
+    TileRadix r;
+    double c = 0.0;
+    if (!tile_radix(M, true, f32, &r, &c) || r.cls == 2) continue;
+    if (best_M == 0 || M * (2.0 * c + 6.0) < best) {
+      best = M * (2.0 * c + 6.0);
+      best_M = M;
+    }
+  }
+  return best_M;
 }
 
 namespace {
@@ -160,13 +178,17 @@ cudaError_t configure_pass(ps_plan_s* p, int pass, int sms) {
   const int nin = packed ? (n + 1) / 2 : n;  // physical points of a line
   const bool zhalf = half && N % 2 == 0 && 2 * nin <= N;
   TileRadix r;
-  if (!tile_radix(N, zhalf, sizeof(T) == 4, &r)) return cudaSuccess;
+  const bool blue = !tile_radix(N, zhalf, sizeof(T) == 4, &r);
+  const int M = blue ? p->blue[al].M : N;  // points of the steps
+  if (blue && (M < 2 * N || !tile_radix(M, true, sizeof(T) == 4, &r) || r.cls == 2)) return cudaSuccess;
+  tl.blue = blue;
   TileArgs& a = tl.a;
-  a.N = N;
+  a.N = M;
+  a.Nt = N;
   a.Ra = r.Ra;
   a.Rm = r.Rm;
   a.Rl = r.Rl;
-  a.NRa = N / r.Ra;
+  a.NRa = M / r.Ra;
   a.Kl = r.Ra * r.Rm;
   a.mRa = div_magic((unsigned)a.Ra);
   a.mRm = div_magic((unsigned)a.Rm);
@@ -174,7 +196,7 @@ cudaError_t configure_pass(ps_plan_s* p, int pass, int sms) {
   a.mNRa = div_magic((unsigned)a.NRa);
   a.mNRm = div_magic((unsigned)(r.Ra * r.Rl));
   a.mKl = div_magic((unsigned)a.Kl);
-  a.tws = L / N;
+  a.tws = blue ? 1 : L / N;
   a.lc = al == 0 ? 1 : 0;
   const int pad = (a.lc && a.NRa % 2 == 0) ? 1 : 0;  // odd stride of digit 1: rows of a step on different banks
   const int row = r.Ra * (a.NRa + pad);
@@ -235,7 +257,7 @@ cudaError_t configure_pass(ps_plan_s* p, int pass, int sms) {
     a.sp_out = so[ap];
     a.se_out = (int)so[al];
     if (si[al] > 0x7fffffffLL || so[al] > 0x7fffffffLL) return cudaSuccess;
-    a.nin = n;
+    a.nin = pass == P4 ? N : n;
     a.nout = pass == P2 ? N : n;
     if (pass == P3) {
       const long long Ks[3] = {1, (long long)p->ldk, (long long)(p->H[1] + 1) * (long long)p->ldk};
@@ -271,7 +293,8 @@ cudaError_t configure_pass(ps_plan_s* p, int pass, int sms) {
   }
   a.elems = row * tk;
   tl.threads = sh.threads;
-  tl.smem = ((size_t)a.elems + N) * sizeof(C);
+  tl.smem = ((size_t)a.elems + M) * sizeof(C);
+  if (blue) tl.fn = tile_blue_kernel<T>(pass, real_pass && !packed);
   // tiles of one plane keep their rows aligned; tiles across planes leave no
   // line slot empty, which pays where the arithmetic bounds the pass (FP64)
   const long long padded = (long long)((a.ntl + tk - 1) / tk) * tk;
@@ -308,7 +331,10 @@ cudaError_t launch_tile(ps_plan_s* p, int pass, const void* src, void* dst, doub
   a.src = a.rsrc = src;
   a.dst = a.rdst = dst;
   a.K = p->K;
-  a.tw = a.twL = p->tw[al];
+  a.twL = p->tw[al];
+  a.tw = tl.blue ? p->blue[al].twM : p->tw[al];
+  a.chirp = p->blue[al].chirp;
+  a.Bf = p->blue[al].Bf;
   a.partials = p->partials;
   a.nparts = z_pass_ctas(p);
   a.escale = 0.5 * p->h * p->h * p->h;

@@ -145,7 +145,7 @@ __device__ __forceinline__ int k_pos(const TileArgs& a, int k) {
   return k1 * a.s1 + k2 * a.s2 + r * a.es;
 }
 
-// first forward step: lines(t)(element) gives the inputs, half of them zero for HALF
+// first forward step: lines(t)(tile address, element) gives the inputs, half of them zero for HALF
 template <int DIR, bool HALF, int CLS, class C, class Ln>
 __device__ __forceinline__ void step_first(const TileArgs& a, const Tile<C>& s, Ln&& lines) {
   radix_switch<CLS, false>(a.Ra, [&](auto rc) {
@@ -154,18 +154,18 @@ __device__ __forceinline__ void step_first(const TileArgs& a, const Tile<C>& s, 
       constexpr int RN = HALF ? R / 2 : R;
       tasks(a, a.NRa, a.mNRa, [&](int t, int b) {
         const auto ld = lines(t);
+        C* p = s.sh + t * a.ls + b * a.es;
         C x[R];
 #pragma unroll
-        for (int r = 0; r < RN; ++r) x[r] = ld(b + r * a.NRa);
+        for (int r = 0; r < RN; ++r) x[r] = ld(p + r * a.s1, b + r * a.NRa);
         dft<R, DIR, full_mask(RN)>(x);
-        C* p = s.sh + t * a.ls + b * a.es;
 #pragma unroll
         for (int r = 0; r < R; ++r) p[r * a.s1] = x[r];
       });
     }
   });
 }
-// final inverse step: lines(t)(element, value) takes the outputs, the lower half for HALF
+// final inverse step: lines(t)(tile address, element, value) takes the outputs, the lower half for HALF
 template <bool HALF, int CLS, class C, class Ln>
 __device__ __forceinline__ void step_final(const TileArgs& a, const Tile<C>& s, Ln&& lines) {
   radix_switch<CLS, false>(a.Ra, [&](auto rc) {
@@ -174,13 +174,13 @@ __device__ __forceinline__ void step_final(const TileArgs& a, const Tile<C>& s, 
       constexpr int RN = HALF ? R / 2 : R;
       tasks(a, a.NRa, a.mNRa, [&](int t, int b) {
         C x[R];
-        const C* p = s.sh + t * a.ls + b * a.es;
+        C* p = s.sh + t * a.ls + b * a.es;
 #pragma unroll
         for (int r = 0; r < R; ++r) x[r] = p[r * a.s1];
         dft_pre<R, 1>(x, s.tw, b, a.NRa);
         const auto st = lines(t);
 #pragma unroll
-        for (int r = 0; r < RN; ++r) st(b + r * a.NRa, x[r]);
+        for (int r = 0; r < RN; ++r) st(p + r * a.s1, b + r * a.NRa, x[r]);
       });
     }
   });
@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_line(const
     step_first<-1, HALF, CLS>(a, s, [&](int t) {
       bool ok;
       const C* src = in(t, &ok);
-      return [&a, src, ok](int e) { return ok && e < a.nin ? src[(long long)e * a.se_in] : mk(T(0), T(0)); };
+      return [&a, src, ok](C*, int e) { return ok && e < a.nin ? src[(long long)e * a.se_in] : mk(T(0), T(0)); };
     });
     steps_sync();
     step_middle<-1, CLS>(a, s);
@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_line(const
     step_final<HALF, CLS>(a, s, [&](int t) {
       bool ok;
       C* dst = out(t, &ok);
-      return [&a, dst, ok](int e, C v) {
+      return [&a, dst, ok](C*, int e, C v) {
         if (ok && e < a.nout) dst[(long long)e * a.se_out] = v;
       };
     });
@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_conv(const
   step_first<-1, HALF, CLS>(a, s, [&](int t) {
     bool ok;
     const C* src = ptr(t, &ok);
-    return [&a, src, ok](int e) { return ok && e < a.nin ? src[(long long)e * a.se_in] : mk(T(0), T(0)); };
+    return [&a, src, ok](C*, int e) { return ok && e < a.nin ? src[(long long)e * a.se_in] : mk(T(0), T(0)); };
   });
   steps_sync();
   step_middle<-1, CLS>(a, s);
@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_conv(const
   step_final<HALF, CLS>(a, s, [&](int t) {
     bool ok;
     C* dst = ptr(t, &ok);
-    return [&a, dst, ok](int e, C v) {
+    return [&a, dst, ok](C*, int e, C v) {
       if (ok && e < a.nout) dst[(long long)e * a.se_out] = v;
     };
   });
@@ -391,53 +391,6 @@ __global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_conv(const
 // else a row of length L = 2 N packed as z[m] = x[2m] + i x[2m+1], untangled by
 //   X[k] = E[k] + W_L^k O[k],  E = (Z[k] + conj Z[N-k]) / 2,  O = -i (Z[k] - conj Z[N-k]) / 2.
 // A line of a pair has its second sequence unless it is the last of an odd number.
-template <typename T, bool PAIR, bool HALF, int CLS>
-__global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_r2c(const __grid_constant__ TileArgs a) {
-  using C = cpx<T>;
-  extern __shared__ __align__(16) unsigned char raw[];
-  const Tile<C> s = tile_setup<C>(a, raw);
-  pdl_wait();
-  step_first<-1, HALF, CLS>(a, s, [&](int t) {
-    int line, pl;
-    const bool ok = line_of(a, t, &line, &pl);
-    const T* src = static_cast<const T*>(a.rsrc) + (pl * a.sp_in + line * a.st_in);
-    const bool two = PAIR && 2 * line + 1 < a.nreal;
-    return [&a, src, ok, two](int e) {
-      C v = mk(T(0), T(0));
-      if (!ok || e >= a.nin) return v;
-      const T* p = src + (long long)e * a.se_in;
-      const bool im = PAIR ? two : 2 * e + 1 < a.nreal;
-      if (a.vec && im) return *reinterpret_cast<const C*>(p);
-      v.x = p[0];
-      if (im) v.y = p[a.im_off];
-      return v;
-    };
-  });
-  steps_sync();
-  step_middle<-1, CLS>(a, s);
-  step_last<CLS>(a, s, [&](int) { return [](C* p, int, C v) { *p = v; }; });
-  __syncthreads();
-  const int N = a.N;
-  tasks(a, N / 2 + 1, a.mout, [&](int t, int k) {
-    int line, pl;
-    if (!line_of(a, t, &line, &pl)) return;
-    const C* z = s.sh + t * a.ls;
-    const C zk = z[k_pos(a, k)];
-    const C zm = z[k_pos(a, k == 0 ? 0 : N - k)];
-    const C e = mk(T(0.5) * (zk.x + zm.x), T(0.5) * (zk.y - zm.y));
-    const C o = mk(T(0.5) * (zk.y + zm.y), T(0.5) * (zm.x - zk.x));
-    C* d = static_cast<C*>(a.dst) + (pl * a.sp_out + line * a.st_out);
-    if constexpr (PAIR) {
-      d[(long long)k * a.se_out] = e;
-      if (2 * line + 1 < a.nreal) d[(long long)k * a.se_out + a.im_c] = o;
-    } else {
-      // outputs k and N - k from the same pair: X[N-k] = conj(E - W^k O)
-      const C wo = mul_w<-1>(o, __ldg(static_cast<const C*>(a.twL) + k));
-      d[k] = cadd(e, wo);
-      if (2 * k != N) d[N - k] = mk(e.x - wo.x, wo.y - e.y);
-    }
-  });
-}
 
 // With the energy the last pass has one CTA more in x (shift = 1), which adds the
 // partials of the fused pass and has no lines: its round trips to L2 would
@@ -450,6 +403,107 @@ __device__ __forceinline__ bool energy_cta(const TileArgs& a) {
   return true;
 }
 
+// element e of line t of a real pass: the pair of reals at src, im_off apart
+template <typename T, bool PAIR>
+struct RealLine {
+  T* p0;
+  bool ok, two;
+  __device__ __forceinline__ RealLine(const TileArgs& a, const void* base, long long sp, long long st, int t) {
+    int line, pl;
+    ok = line_of(a, t, &line, &pl);
+    p0 = const_cast<T*>(static_cast<const T*>(base)) + (pl * sp + line * st);
+    two = PAIR && 2 * line + 1 < a.nreal;
+  }
+  __device__ __forceinline__ cpx<T> load(const TileArgs& a, int e) const {
+    cpx<T> v = mk(T(0), T(0));
+    if (!ok || e >= a.nin) return v;
+    const T* p = p0 + (long long)e * a.se_in;
+    const bool im = PAIR ? two : 2 * e + 1 < a.nreal;
+    if (a.vec && im) return *reinterpret_cast<const cpx<T>*>(p);
+    v.x = p[0];
+    if (im) v.y = p[a.im_off];
+    return v;
+  }
+  __device__ __forceinline__ void store(const TileArgs& a, int e, cpx<T> v) const {
+    if (!ok || e >= a.nout) return;
+    T* p = p0 + (long long)e * a.se_out;
+    const bool im = PAIR ? two : 2 * e + 1 < a.nreal;
+    if (a.vec && im) {
+      *reinterpret_cast<cpx<T>*>(p) = v;
+    } else {
+      p[0] = v.x;
+      if (im) p[a.im_off] = v.y;
+    }
+  }
+};
+
+// the outputs of line t of a forward real pass at wavenumber k from Z[k], Z[N-k]
+template <typename T, bool PAIR>
+__device__ __forceinline__ void untangle(const TileArgs& a, int t, int k, int N, cpx<T> zk, cpx<T> zm) {
+  using C = cpx<T>;
+  int line, pl;
+  if (!line_of(a, t, &line, &pl)) return;
+  const C e = mk(T(0.5) * (zk.x + zm.x), T(0.5) * (zk.y - zm.y));
+  const C o = mk(T(0.5) * (zk.y + zm.y), T(0.5) * (zm.x - zk.x));
+  C* d = static_cast<C*>(a.dst) + (pl * a.sp_out + line * a.st_out);
+  if constexpr (PAIR) {
+    d[(long long)k * a.se_out] = e;
+    if (2 * line + 1 < a.nreal) d[(long long)k * a.se_out + a.im_c] = o;
+  } else {
+    // outputs k and N - k from the same pair: X[N-k] = conj(E - W^k O)
+    const C wo = mul_w<-1>(o, __ldg(static_cast<const C*>(a.twL) + k));
+    d[k] = cadd(e, wo);
+    if (2 * k != N) d[N - k] = mk(e.x - wo.x, wo.y - e.y);
+  }
+}
+
+// Z[k] and Z[N-k] of line t of an inverse real pass
+template <typename T, bool PAIR>
+__device__ __forceinline__ void tangle(const TileArgs& a, int t, int k, int N, cpx<T>* zk, cpx<T>* zm) {
+  using C = cpx<T>;
+  int line, pl;
+  *zk = *zm = mk(T(0), T(0));
+  if (!line_of(a, t, &line, &pl)) return;
+  const C* x = static_cast<const C*>(a.src) + (pl * a.sp_in + line * a.st_in);
+  if constexpr (PAIR) {
+    // Z[k] = A + i B, Z[N-k] = conj A + i conj B; A and B are real at k = 0 and
+    // N/2, so their (rounding-level) imaginary parts there are dropped
+    C A = x[(long long)k * a.se_in], B = mk(T(0), T(0));
+    if (2 * line + 1 < a.nreal) B = x[(long long)k * a.se_in + a.im_c];
+    if (k == 0 || 2 * k == N) A.y = B.y = T(0);
+    *zk = mk(A.x - B.y, A.y + B.x);
+    *zm = mk(A.x + B.y, B.x - A.y);
+  } else {
+    // Z[k] = E' + i O', E' = X[k] + conj X[N-k], O' = (X[k] - conj X[N-k]) conj W_L^k;
+    // E'[N-k] = conj E'[k], O'[N-k] = conj O'[k]
+    const C xk = x[k], xm = x[N - k];
+    const C e = mk(xk.x + xm.x, xk.y - xm.y);
+    const C o = mul_w<1>(mk(xk.x - xm.x, xk.y + xm.y), __ldg(static_cast<const C*>(a.twL) + k));
+    *zk = mk(e.x - o.y, e.y + o.x);
+    *zm = mk(e.x + o.y, o.x - e.y);
+  }
+}
+
+template <typename T, bool PAIR, bool HALF, int CLS>
+__global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_r2c(const __grid_constant__ TileArgs a) {
+  using C = cpx<T>;
+  extern __shared__ __align__(16) unsigned char raw[];
+  const Tile<C> s = tile_setup<C>(a, raw);
+  pdl_wait();
+  step_first<-1, HALF, CLS>(a, s, [&](int t) {
+    const RealLine<T, PAIR> r(a, a.rsrc, a.sp_in, a.st_in, t);
+    return [&a, r](C*, int e) { return r.load(a, e); };
+  });
+  steps_sync();
+  step_middle<-1, CLS>(a, s);
+  step_last<CLS>(a, s, [&](int) { return [](C* p, int, C v) { *p = v; }; });
+  __syncthreads();
+  tasks(a, a.N / 2 + 1, a.mout, [&](int t, int k) {
+    const C* z = s.sh + t * a.ls;
+    untangle<T, PAIR>(a, t, k, a.N, z[k_pos(a, k)], z[k_pos(a, k == 0 ? 0 : a.N - k)]);
+  });
+}
+
 template <typename T, bool PAIR, bool HALF, int CLS>
 __global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_c2r(const __grid_constant__ TileArgs a) {
   using C = cpx<T>;
@@ -460,28 +514,8 @@ __global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_c2r(const 
   pdl_wait();
   // Z[k] and Z[N-k] from the same pair of inputs
   tasks(a, N / 2 + 1, a.mout, [&](int t, int k) {
-    int line, pl;
-    C zk = mk(T(0), T(0)), zm = zk;
-    if (line_of(a, t, &line, &pl)) {
-      const C* x = static_cast<const C*>(a.src) + (pl * a.sp_in + line * a.st_in);
-      if constexpr (PAIR) {
-        // Z[k] = A + i B, Z[N-k] = conj A + i conj B; A and B are real at k = 0 and
-        // N/2, so their (rounding-level) imaginary parts there are dropped
-        C A = x[(long long)k * a.se_in], B = zk;
-        if (2 * line + 1 < a.nreal) B = x[(long long)k * a.se_in + a.im_c];
-        if (k == 0 || 2 * k == N) A.y = B.y = T(0);
-        zk = mk(A.x - B.y, A.y + B.x);
-        zm = mk(A.x + B.y, B.x - A.y);
-      } else {
-        // Z[k] = E' + i O', E' = X[k] + conj X[N-k], O' = (X[k] - conj X[N-k]) conj W_L^k;
-        // E'[N-k] = conj E'[k], O'[N-k] = conj O'[k]
-        const C xk = x[k], xm = x[N - k];
-        const C e = mk(xk.x + xm.x, xk.y - xm.y);
-        const C o = mul_w<1>(mk(xk.x - xm.x, xk.y + xm.y), __ldg(static_cast<const C*>(a.twL) + k));
-        zk = mk(e.x - o.y, e.y + o.x);
-        zm = mk(e.x + o.y, o.x - e.y);
-      }
-    }
+    C zk, zm;
+    tangle<T, PAIR>(a, t, k, N, &zk, &zm);
     C* z = s.sh + t * a.ls;
     z[k_pos(a, k)] = zk;
     if (k != 0 && 2 * k != N) z[k_pos(a, N - k)] = zm;
@@ -491,22 +525,219 @@ __global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_c2r(const 
   steps_sync();
   step_middle<1, CLS>(a, s);
   step_final<HALF, CLS>(a, s, [&](int t) {
+    const RealLine<T, PAIR> r(a, a.rdst, a.sp_out, a.st_out, t);
+    return [&a, r](C*, int e, C v) { r.store(a, e, v); };
+  });
+}
+
+// ------------------------------------------------------------ Bluestein form
+
+// Lines whose length N has a prime factor above 31 (or two above 16): the chirp-z
+// form X[k] = c[k] sum_m (x[m] c[m]) conj(c[k-m]), c[m] = exp(-i pi m^2 / N), as a
+// cyclic convolution of length M >= 2 N on the steps above (a.N = M, a.Nt = N):
+// the chirp product in the loads, the product with the transformed conjugate chirp Bf
+// between the last forward and the first inverse step, the chirp again in the
+// stores. DIR = +1 conjugates the chirp and Bf.
+
+template <int DIR, int CLS, class C>
+__device__ __forceinline__ void blue_multiply(const TileArgs& a, const Tile<C>& s) {
+  radix_switch<CLS, true>(a.Rl, [&](auto rc) {
+    constexpr int R = rc;
+    tasks(a, a.Kl, a.mKl, [&](int t, int b) {
+      int pos, e;
+      last_digits(a, b, &pos, &e);
+      C* p = s.sh + t * a.ls + pos;
+      C x[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) x[r] = p[r * a.es];
+      dft_pre<R, -1>(x, s.tw, e, a.Kl);
+#pragma unroll
+      for (int r = 0; r < R; ++r) x[r] = mul_w<DIR>(x[r], __ldg(static_cast<const C*>(a.Bf) + e + r * a.Kl));
+      dft<R, 1, full_mask(R)>(x);
+#pragma unroll
+      for (int r = 0; r < R; ++r) p[r * a.es] = x[r];
+    });
+  });
+  __syncthreads();
+}
+// the whole convolution: ld and st as of step_first and step_final, with chirps
+template <int DIR, int CLS, class C, class Ld, class St>
+__device__ __forceinline__ void blue_conv(const TileArgs& a, const Tile<C>& s, Ld&& ld, St&& st) {
+  step_first<-1, true, CLS>(a, s, ld);
+  steps_sync();
+  step_middle<-1, CLS>(a, s);
+  blue_multiply<DIR, CLS>(a, s);
+  step_middle<1, CLS>(a, s);
+  step_final<true, CLS>(a, s, st);
+}
+template <class C>
+__device__ __forceinline__ C chirp(const TileArgs& a, int m) { return __ldg(static_cast<const C*>(a.chirp) + m); }
+// tile position of element m before the first and after the final step
+__device__ __forceinline__ int n_pos(const TileArgs& a, int m) {
+  const int n1 = div_by(m, a.mNRa);
+  return n1 * a.s1 + (m - n1 * a.NRa) * a.es;
+}
+
+template <typename T, int DIR, int CLS>
+__global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_blue_line(const __grid_constant__ TileArgs a) {
+  using C = cpx<T>;
+  extern __shared__ __align__(16) unsigned char raw[];
+  const Tile<C> s = tile_setup<C>(a, raw);
+  pdl_wait();
+  blue_conv<DIR, CLS>(
+      a, s,
+      [&](int t) {
+        int line, pl;
+        const bool ok = line_of(a, t, &line, &pl);
+        const C* src = static_cast<const C*>(a.src) + (pl * a.sp_in + line * a.st_in);
+        return [&a, src, ok](C*, int e) {
+          return ok && e < a.nin ? mul_w<DIR>(src[(long long)e * a.se_in], chirp<C>(a, e)) : mk(T(0), T(0));
+        };
+      },
+      [&](int t) {
+        int line, pl;
+        const bool ok = line_of(a, t, &line, &pl);
+        C* dst = static_cast<C*>(a.dst) + (pl * a.sp_out + line * a.st_out);
+        return [&a, dst, ok](C*, int e, C v) {
+          if (ok && e < a.nout) dst[(long long)e * a.se_out] = mul_w<DIR>(v, chirp<C>(a, e));
+        };
+      });
+}
+
+// Forward, K^F, inverse: between the two convolutions the chirps cancel (|c| = 1), so
+// u[k] = K[k] v[k] of the first one's values v is the second one's input, and
+// |X|^2 = |v|^2 in the energy; the final step of the first and the first step of the
+// second share their elements.
+template <typename T, int CLS>
+__global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_blue_conv(const __grid_constant__ TileArgs a) {
+  using C = cpx<T>;
+  extern __shared__ __align__(16) unsigned char raw[];
+  __shared__ T wsum[8];
+  const Tile<C> s = tile_setup<C>(a, raw);
+  auto at = [&](int t, int* line, int* pl) {
+    const bool ok = line_of(a, t, line, pl);
+    if (a.pair_pl && ok) *pl = paired_ky(*pl, a.npl);
+    return ok;
+  };
+  auto ptr = [&](int t, bool* ok) {
     int line, pl;
-    const bool ok = line_of(a, t, &line, &pl);
-    T* dst = static_cast<T*>(a.rdst) + (pl * a.sp_out + line * a.st_out);
-    const bool two = PAIR && 2 * line + 1 < a.nreal;
-    return [&a, dst, ok, two](int e, C v) {
-      if (!ok || e >= a.nout) return;
-      T* p = dst + (long long)e * a.se_out;
-      const bool im = PAIR ? two : 2 * e + 1 < a.nreal;
-      if (a.vec && im) {
-        *reinterpret_cast<C*>(p) = v;
-      } else {
-        p[0] = v.x;
-        if (im) p[a.im_off] = v.y;
-      }
+    *ok = at(t, &line, &pl);
+    return static_cast<C*>(a.dst) + (pl * a.sp_in + line * a.st_in);
+  };
+  pdl_wait();
+  step_first<-1, true, CLS>(a, s, [&](int t) {
+    bool ok;
+    const C* src = ptr(t, &ok);
+    return [&a, src, ok](C*, int e) {
+      return ok && e < a.nin ? mul_w<-1>(src[(long long)e * a.se_in], chirp<C>(a, e)) : mk(T(0), T(0));
     };
   });
+  steps_sync();
+  step_middle<-1, CLS>(a, s);
+  blue_multiply<-1, CLS>(a, s);
+  step_middle<1, CLS>(a, s);
+  T en = T(0);
+  radix_switch<CLS, false>(a.Ra, [&](auto rc) {
+    constexpr int R = rc;
+    if constexpr (R % 2 == 0) {
+      tasks(a, a.NRa, a.mNRa, [&](int t, int b) {
+        int line, pl;
+        const bool ok = at(t, &line, &pl);
+        const T* Kp = static_cast<const T*>(a.K) + (long long)min(pl, a.Lp - pl) * a.Ksp +
+                      (long long)min(line, a.Lt - line) * a.Kst;
+        C* p = s.sh + t * a.ls + b * a.es;
+        C x[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) x[r] = p[r * a.s1];
+        dft_pre<R, 1>(x, s.tw, b, a.NRa);
+        T el = T(0);
+#pragma unroll
+        for (int r = 0; r < R / 2; ++r) {
+          const int k = b + r * a.NRa;
+          const T kk = ok && k < a.Nt ? __ldg(Kp + (long long)min(k, a.Nt - k) * a.Kse) : T(0);
+          const C u = mk(kk * x[r].x, kk * x[r].y);
+          el = mad(u.x, x[r].x, mad(u.y, x[r].y, el));
+          x[r] = u;
+        }
+        const int k0 = a.w_tile ? line : pl;
+        en = mad(k0 == 0 || 2 * k0 == a.La0 ? T(1) : T(2), el, en);
+        dft<R, -1, full_mask(R / 2)>(x);
+#pragma unroll
+        for (int r = 0; r < R; ++r) p[r * a.s1] = x[r];
+      });
+    }
+  });
+  if (a.E != nullptr) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) en += __shfl_xor_sync(0xffffffffu, en, o);
+    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = en;
+  }
+  __syncthreads();
+  if (a.E != nullptr && threadIdx.x == 0) {
+    double sum = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) sum += (double)wsum[w];
+    a.partials[blockIdx.y * gridDim.x + blockIdx.x] = sum;
+  }
+  step_middle<-1, CLS>(a, s);
+  blue_multiply<1, CLS>(a, s);
+  step_middle<1, CLS>(a, s);
+  step_final<true, CLS>(a, s, [&](int t) {
+    bool ok;
+    C* dst = ptr(t, &ok);
+    return [&a, dst, ok](C*, int e, C v) {
+      if (ok && e < a.nout) dst[(long long)e * a.se_out] = mul_w<1>(v, chirp<C>(a, e));
+    };
+  });
+}
+
+template <typename T, bool PAIR, int CLS>
+__global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_blue_r2c(const __grid_constant__ TileArgs a) {
+  using C = cpx<T>;
+  extern __shared__ __align__(16) unsigned char raw[];
+  const Tile<C> s = tile_setup<C>(a, raw);
+  pdl_wait();
+  blue_conv<-1, CLS>(
+      a, s,
+      [&](int t) {
+        const RealLine<T, PAIR> r(a, a.rsrc, a.sp_in, a.st_in, t);
+        return [&a, r](C*, int e) { return e < a.nin ? mul_w<-1>(r.load(a, e), chirp<C>(a, e)) : mk(T(0), T(0)); };
+      },
+      [&](int) {
+        return [&a](C* p, int e, C v) {
+          if (e < a.Nt) *p = mul_w<-1>(v, chirp<C>(a, e));
+        };
+      });
+  __syncthreads();
+  tasks(a, a.Nt / 2 + 1, a.mout, [&](int t, int k) {
+    const C* z = s.sh + t * a.ls;
+    untangle<T, PAIR>(a, t, k, a.Nt, z[n_pos(a, k)], z[n_pos(a, k == 0 ? 0 : a.Nt - k)]);
+  });
+}
+
+template <typename T, bool PAIR, int CLS>
+__global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_blue_c2r(const __grid_constant__ TileArgs a) {
+  using C = cpx<T>;
+  extern __shared__ __align__(16) unsigned char raw[];
+  if (energy_cta(a)) return;
+  const Tile<C> s = tile_setup<C>(a, raw);
+  const int N = a.Nt;
+  pdl_wait();
+  tasks(a, N / 2 + 1, a.mout, [&](int t, int k) {
+    C zk, zm;
+    tangle<T, PAIR>(a, t, k, N, &zk, &zm);
+    C* z = s.sh + t * a.ls;
+    z[n_pos(a, k)] = mul_w<1>(zk, chirp<C>(a, k));
+    if (k != 0 && 2 * k != N) z[n_pos(a, N - k)] = mul_w<1>(zm, chirp<C>(a, N - k));
+  });
+  __syncthreads();
+  blue_conv<1, CLS>(
+      a, s, [&](int) { return [&a](C* p, int e) { return e < a.Nt ? *p : mk(T(0), T(0)); }; },
+      [&](int t) {
+        const RealLine<T, PAIR> r(a, a.rdst, a.sp_out, a.st_out, t);
+        return [&a, r](C*, int e, C v) {
+          if (e < a.nout) r.store(a, e, mul_w<1>(v, chirp<C>(a, e)));
+        };
+      });
 }
 
 }  // namespace tile

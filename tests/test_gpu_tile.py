@@ -14,9 +14,11 @@ TOL = {"f64": 1e-12, "f32": 1e-5}
 
 # 4 = 2 x 2 is the shortest; 26, 33, 91, 169 use 11 and 13; 343 and 2197 three odd
 # steps; 2000 and 4096 the longest tables; the others mix the composite radices;
-# the second row ends in a prime radix from 17 to 31, behind one step, two or none
+# the second row ends in a prime radix from 17 to 31, behind one step, two or none; the
+# third runs in Bluestein form
 LENGTHS = [4, 6, 9, 15, 22, 26, 33, 63, 70, 90, 91, 126, 150, 169, 208, 220, 231, 343, 420, 1000, 2000, 2197, 4096,
-           17, 19, 31, 34, 46, 62, 93, 116, 221, 247, 406, 1085, 1472]
+           17, 19, 31, 34, 46, 62, 93, 116, 221, 247, 406, 1085, 1472,
+           37, 74, 106, 127, 289, 323, 487, 578, 1022, 1031]
 
 
 @pytest.mark.parametrize("dtype", ["f64", "f32"])
