@@ -15,14 +15,57 @@
 // kernel: the inverse's first step needs exactly the k1 values the forward's
 // last step left in each thread, so the spectrum never leaves registers.
 #include "fft_fast.cuh"
+#include "fft_regs.cuh"
 #include "reduce.cuh"
 #include "tile_dft.cuh"
 
 namespace ps {
 
+using regs::rdft;
 using tile::dft;
 using tile::dft_pre;
 using tile::full_mask;
+
+// The four transforms of a line: columns b forward (P points over a, then the twiddles
+// W_L^{b k1}), rows k1 forward and inverse (Q points), columns inverse (the
+// conjugate twiddles, then P points). At L = 1024 the twiddles are folded into the
+// radix-2 layers of the transform that follows them (480 operations for 32 points behind
+// twiddles instead of about 570; the z pass at 512^3 2202 -> 2158 us, the inverse y
+// pass 579 -> 564 us); the shorter lengths gain no time by it and keep the
+// separate products, whose rounding error is a little smaller.
+template <int P, int Q>
+constexpr bool kFold = P * Q >= 1024;
+
+template <int P, int Q, bool HALF>
+__device__ __forceinline__ void col_fwd(float2 (&y)[P], const float2* tw, int b) {
+  if constexpr (kFold<P, Q>) {
+    dft<P, -1, full_mask(HALF ? P / 2 : P)>(y);
+  } else {
+    rdft<P, -1, HALF>(y);
+#pragma unroll
+    for (int k1 = 1; k1 < P; ++k1) y[k1] = cmul(y[k1], tw[b * k1]);
+  }
+}
+template <int P, int Q>
+__device__ __forceinline__ void row_fwd(float2 (&x)[Q], const float2* tw, int k1) {
+  if constexpr (kFold<P, Q>) dft_pre<Q, -1>(x, tw, k1, P);
+  else rdft<Q, -1, false>(x);
+}
+template <int P, int Q>
+__device__ __forceinline__ void row_inv(float2 (&x)[Q], const float2* tw, int k1) {
+  if constexpr (kFold<P, Q>) {
+    dft<Q, 1, full_mask(Q)>(x);
+  } else {
+    rdft<Q, 1, false>(x);
+#pragma unroll
+    for (int b = 1; b < Q; ++b) x[b] = cmulc(x[b], tw[b * k1]);
+  }
+}
+template <int P, int Q>
+__device__ __forceinline__ void col_inv(float2 (&y)[P], const float2* tw, int b) {
+  if constexpr (kFold<P, Q>) dft_pre<P, 1>(y, tw, b, Q);
+  else rdft<P, 1, false>(y);
+}
 
 constexpr int kTK = 16;  // lines per CTA
 
@@ -67,7 +110,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q),
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
       const int b = j + T * u;
-      dft<P, -1, full_mask(NA)>(y[u]);
+      col_fwd<P, Q, HALF>(y[u], tw, b);
 #pragma unroll
       for (int k1 = 0; k1 < P; ++k1) sh[(b * P + k1) * TK + t] = y[u][k1];
     }
@@ -77,7 +120,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q),
       const int k1 = j + T * v;
 #pragma unroll
       for (int b = 0; b < Q; ++b) X[v][b] = sh[(b * P + k1) * TK + t];
-      dft_pre<Q, -1>(X[v], tw, k1, P);
+      row_fwd<P, Q>(X[v], tw, k1);
     }
   } else {
 #pragma unroll
@@ -124,10 +167,8 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q),
     // inverse: Q-point transforms over k2, exchange, conjugate twiddles and
     // P-point transforms over k1
 #pragma unroll
-    for (int v = 0; v < NK; ++v) {
-      dft<Q, 1, full_mask(Q)>(X[v]);
-    }
-    if constexpr (KIND == 2) __syncthreads();  // the forward exchange has been read
+    for (int v = 0; v < NK; ++v) row_inv<P, Q>(X[v], tw, j + T * v);
+    // (KIND 2: back to the slots this thread read its rows from, no barrier before)
 #pragma unroll
     for (int v = 0; v < NK; ++v) {
       const int k1 = j + T * v;
@@ -141,7 +182,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q),
       float2 y[P];
 #pragma unroll
       for (int k1 = 0; k1 < P; ++k1) y[k1] = sh[(b * P + k1) * TK + t];
-      dft_pre<P, 1>(y, tw, b, Q);
+      col_inv<P, Q>(y, tw, b);
       if (valid) {
 #pragma unroll
         for (int aa = 0; aa < NA; ++aa)
@@ -302,7 +343,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
       const int b = j + T * u;
-      dft<P, -1, full_mask(NA)>(y[u]);
+      col_fwd<P, Q, HALF>(y[u], tws, b);
 #pragma unroll
       for (int k1 = 0; k1 < P; ++k1) sh[(b * PP + k1) * TK + t] = y[u][k1];
     }
@@ -314,7 +355,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
       const int k1 = j + T * v;
 #pragma unroll
       for (int b = 0; b < Q; ++b) X[v][b] = sh[(b * PP + k1) * TK + t];
-      dft_pre<Q, -1>(X[v], tws, k1, P);
+      row_fwd<P, Q>(X[v], tws, k1);
       // V^F = K^F rho^F on the even octant of K^F; energy sum K |rho^F|^2
 #pragma unroll
       for (int k2 = 0; k2 < Q; ++k2) {
@@ -325,19 +366,19 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
         e1 = fmaf(kk, x.x * x.x + x.y * x.y, e1);
         X[v][k2] = make_float2(kk * x.x, kk * x.y);
       }
-      dft<Q, 1, full_mask(Q)>(X[v]);
+      row_inv<P, Q>(X[v], tws, k1);
     }
     eacc += e1 * ((kx == 0 || 2 * kx == a.L1) ? 1.f : 2.f);
-    __syncthreads();  // the forward exchange and the K^F slice have been read
-    if (next < ntiles) issue_k(nkt, nyi);
-    cp_async_commit();
+    // back to the slots this thread read its rows from: no barrier before
 #pragma unroll
     for (int v = 0; v < NK; ++v) {
       const int k1 = j + T * v;
 #pragma unroll
       for (int b = 0; b < Q; ++b) sh[(b * PP + k1) * TK + t] = X[v][b];
     }
-    __syncthreads();
+    __syncthreads();  // the K^F slice has been read too
+    if (next < ntiles) issue_k(nkt, nyi);
+    cp_async_commit();
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
       const int b = j + T * u;
@@ -350,7 +391,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
       const int b = j + T * u;
-      dft_pre<P, 1>(y[u], tws, b, Q);
+      col_inv<P, Q>(y[u], tws, b);
       if (valid) {
 #pragma unroll
         for (int aa = 0; aa < NA; ++aa)
@@ -489,7 +530,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
 #pragma unroll
       for (int u = 0; u < NB; ++u) {
         const int b = j + T * u;
-        dft<P, -1, full_mask(NA)>(y[u]);
+        col_fwd<P, Q, HALF>(y[u], tw, b);
 #pragma unroll
         for (int k1 = 0; k1 < P; ++k1) sh[(b * PP + k1) * TK + t] = y[u][k1];
       }
@@ -506,7 +547,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
 #pragma unroll
       for (int v = 0; v < NK; ++v) {
         const int k1 = j + T * v;
-        dft_pre<Q, -1>(X[v], tw, k1, P);
+        row_fwd<P, Q>(X[v], tw, k1);
         if (valid) {
 #pragma unroll
           for (int k2 = 0; k2 < Q; ++k2) d[(long long)(k1 + P * k2) * a.dst_elem] = X[v][k2];
@@ -524,7 +565,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
 #pragma unroll
       for (int v = 0; v < NK; ++v) {
         const int k1 = j + T * v;
-        dft<Q, 1, full_mask(Q)>(X[v]);
+        row_inv<P, Q>(X[v], tw, k1);
 #pragma unroll
         for (int b = 0; b < Q; ++b) sh[(b * PP + k1) * TK + t] = X[v][b];
       }
@@ -542,7 +583,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
 #pragma unroll
       for (int u = 0; u < NB; ++u) {
         const int b = j + T * u;
-        dft_pre<P, 1>(y[u], tw, b, Q);
+        col_inv<P, Q>(y[u], tw, b);
         if (valid) {
 #pragma unroll
           for (int aa = 0; aa < NA; ++aa)
