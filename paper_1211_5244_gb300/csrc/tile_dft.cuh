@@ -159,10 +159,8 @@ __device__ __forceinline__ C mul_w(C v, C w) {
 // ------------------------------------------------------------ transforms
 
 // powers of two: radix-2 decimation in time, layer by layer on bit-reversed inputs
-template <int R, int DIR, Mask MASK, class C>
-__device__ __forceinline__ void dft_pow2(C (&x)[R]) {
-  C y[R];
-  sfor<R>([&](auto i) { y[bitrev(i, R)] = x[i]; });
+template <int R, int DIR, Mask MASK, int FROM, class C>
+__device__ __forceinline__ void pow2_layers(C (&y)[R]) {  // layers of blocks of FROM .. R points
   auto layer = [&](auto mc) {
     constexpr int m = mc;
     sfor<R / m>([&](auto blk) {
@@ -181,16 +179,60 @@ __device__ __forceinline__ void dft_pow2(C (&x)[R]) {
       });
     });
   };
-  if constexpr (R >= 2) layer(std::integral_constant<int, 2>{});
-  if constexpr (R >= 4) layer(std::integral_constant<int, 4>{});
+  if constexpr (FROM <= 2 && R >= 2) layer(std::integral_constant<int, 2>{});
+  if constexpr (FROM <= 4 && R >= 4) layer(std::integral_constant<int, 4>{});
   if constexpr (R >= 8) layer(std::integral_constant<int, 8>{});
   if constexpr (R >= 16) layer(std::integral_constant<int, 16>{});
   if constexpr (R >= 32) layer(std::integral_constant<int, 32>{});
+}
+template <int R, int DIR, Mask MASK, class C>
+__device__ __forceinline__ void dft_pow2(C (&x)[R]) {
+  C y[R];
+  sfor<R>([&](auto i) { y[bitrev(i, R)] = x[i]; });
+  pow2_layers<R, DIR, MASK, 2>(y);
   sfor<R>([&](auto i) { x[i] = y[i]; });
 }
 
 // odd primes: y_m, y_{p-m} = t_m +- DIR i u_m with t_m = x_0 + sum_k cos(2 pi m k / p) a_k,
-// u_m = sum_k sin(2 pi m k / p) b_k, a_k, b_k = x_k +- x_{p-k}, k = 1 .. (p-1)/2
+// u_m = sum_k sin(2 pi m k / p) b_k, a_k, b_k = x_k +- x_{p-k}, k = 1 .. (p-1)/2. From p = 5 on
+// y_m is one chain of FMAs from t_m and y_{p-m} = 2 t_m - y_m, an operation less per
+// component than forming u_m (5 points: 32 operations instead of 36).
+template <int P, int DIR, Mask MASK, class C>
+__device__ __forceinline__ void prime_pairs(C (&x)[P], C x0, const C (&a)[(P - 1) / 2], const C (&b)[(P - 1) / 2]) {
+  using S = decltype(x0.x);
+  constexpr int H = (P - 1) / 2;
+  C sum = x0;
+  sfor<H>([&](auto kc) {
+    if constexpr (((MASK >> (kc + 1)) | (MASK >> (P - kc - 1))) & 1) sum = cadd(sum, a[kc]);
+  });
+  C y[P];
+  y[0] = sum;
+  sfor<H>([&](auto mc) {
+    constexpr int m = mc + 1;
+    C t = x0;
+    sfor<H>([&](auto kc) {
+      constexpr int k = kc + 1;
+      if constexpr (((MASK >> k) | (MASK >> (P - k))) & 1) {
+        constexpr S c = (S)cos_turn(m * k, P);
+        t = mk(mad(c, a[kc].x, t.x), mad(c, a[kc].y, t.y));
+      }
+    });
+    C v = t, w = t;  // t +- DIR i u
+    sfor<H>([&](auto kc) {
+      constexpr int k = kc + 1;
+      if constexpr (((MASK >> k) | (MASK >> (P - k))) & 1) {
+        constexpr S s = (S)(DIR * sin_turn(m * k, P));
+        v = mk(mad(-s, b[kc].y, v.x), mad(s, b[kc].x, v.y));
+        if constexpr (H == 1) w = mk(mad(s, b[kc].y, w.x), mad(-s, b[kc].x, w.y));
+      }
+    });
+    if constexpr (H > 1) w = mk(mad(S(2), t.x, -v.x), mad(S(2), t.y, -v.y));
+    y[m] = v;
+    y[P - m] = w;
+  });
+  sfor<P>([&](auto i) { x[i] = y[i]; });
+}
+
 template <int P, int DIR, Mask MASK, class C>
 __device__ __forceinline__ void dft_prime(C (&x)[P]) {
   using S = decltype(x[0].x);
@@ -209,28 +251,7 @@ __device__ __forceinline__ void dft_prime(C (&x)[P]) {
       b[k - 1] = mk(-x[P - k].x, -x[P - k].y);
     }
   });
-  const C x0 = (MASK & 1) ? x[0] : mk(S(0), S(0));
-  C sum = x0;
-  sfor<H>([&](auto kc) {
-    if constexpr (((MASK >> (kc + 1)) | (MASK >> (P - kc - 1))) & 1) sum = cadd(sum, a[kc]);
-  });
-  C y[P];
-  y[0] = sum;
-  sfor<H>([&](auto mc) {
-    constexpr int m = mc + 1;
-    C t = x0, u = mk(S(0), S(0));
-    sfor<H>([&](auto kc) {
-      constexpr int k = kc + 1;
-      if constexpr (((MASK >> k) | (MASK >> (P - k))) & 1) {
-        constexpr S c = (S)cos_turn(m * k, P), s = (S)(DIR * sin_turn(m * k, P));
-        t = mk(mad(c, a[kc].x, t.x), mad(c, a[kc].y, t.y));
-        u = mk(mad(-s, b[kc].y, u.x), mad(s, b[kc].x, u.y));  // DIR i u
-      }
-    });
-    y[m] = cadd(t, u);
-    y[P - m] = csub(t, u);
-  });
-  sfor<P>([&](auto i) { x[i] = y[i]; });
+  prime_pairs<P, DIR, MASK>(x, (MASK & 1) ? x[0] : mk(S(0), S(0)), a, b);
 }
 
 template <int R, int DIR, Mask MASK, class C>
@@ -271,9 +292,48 @@ __device__ __forceinline__ void dft(C (&x)[R]) {
   }
 }
 
+// The transform of x[r] w(r) (conj(w(r)) for DIR = +1), A a power of two or a prime;
+// w(0) = 1 unless W0. The first additions take pairs p +- w x of a twiddled p, five
+// operations per component instead of six.
+template <int A, int DIR, bool W0, class C, class W>
+__device__ __forceinline__ void dft_tw(C (&x)[A], W&& w) {
+  using S = decltype(x[0].x);
+  auto first = [&](auto r) {
+    if constexpr (r > 0 || W0) return mul_w<DIR>(x[r], w(r));
+    else return x[r];
+  };
+  auto pair = [&](auto r, auto q, C& s, C& d) {  // w(r) x[r] +- w(q) x[q]
+    s = first(r);
+    d = x[q];
+    const C f = w(q);
+    bfly_w(s, d, f.x, DIR < 0 ? f.y : -f.y);
+  };
+  if constexpr ((A & (A - 1)) == 0) {
+    C y[A];
+    sfor<A / 2>([&](auto i) {
+      constexpr int r = bitrev(2 * i, A);
+      pair(std::integral_constant<int, r>{}, std::integral_constant<int, r + A / 2>{}, y[2 * i], y[2 * i + 1]);
+    });
+    pow2_layers<A, DIR, full_mask(A), 4>(y);
+    sfor<A>([&](auto i) { x[i] = y[i]; });
+  } else if constexpr (low_prime(A) == A) {
+    constexpr int H = (A - 1) / 2;
+    C a[H], b[H];
+    sfor<H>([&](auto k) {
+      pair(std::integral_constant<int, k + 1>{}, std::integral_constant<int, A - 1 - k>{}, a[k], b[k]);
+    });
+    const C x0 = first(std::integral_constant<int, 0>{});
+    prime_pairs<A, DIR, full_mask(A)>(x, x0, a, b);
+  } else {
+    sfor<A>([&](auto r) { x[r] = first(r); });
+    dft<A, DIR, full_mask(A)>(x);
+  }
+}
+
 template <int R, int DIR, class C>
 __device__ __forceinline__ void dft_pre(C (&x)[R], const C* tw, int e, int NR) {
-  if constexpr (R > 1 && (R & (R - 1)) == 0) {
+  if constexpr (R == 1) {
+  } else if constexpr ((R & (R - 1)) == 0) {
     C y[R];
     sfor<R>([&](auto i) { y[bitrev(i, R)] = x[i]; });
     auto layer = [&](auto mc) {
@@ -293,11 +353,28 @@ __device__ __forceinline__ void dft_pre(C (&x)[R], const C* tw, int e, int NR) {
     if constexpr (R >= 16) layer(std::integral_constant<int, 16>{});
     if constexpr (R >= 32) layer(std::integral_constant<int, 32>{});
     sfor<R>([&](auto i) { x[i] = y[i]; });
+  } else if constexpr (low_prime(R) == R) {
+    dft_tw<R, DIR, false>(x, [&](auto r) { return tw[e * r]; });
   } else {
-    sfor<R>([&](auto r) {
-      if constexpr (r > 0) x[r] = mul_w<DIR>(x[r], tw[e * r]);
+    // as dft(), with the twiddles in the columns
+    constexpr bool coprime = low_part(R) < R;
+    constexpr int A = coprime ? low_part(R) : R / low_prime(R), B = R / A;
+    constexpr int sn1 = B, sn2 = coprime ? A : 1;
+    constexpr int sk1 = coprime ? B * inv_mod(B % A, A) : 1, sk2 = coprime ? A * inv_mod(A % B, B) : A;
+    C z[B][A];
+    sfor<B>([&](auto n2) {
+      sfor<A>([&](auto n1) { z[n2][n1] = x[(sn1 * n1 + sn2 * n2) % R]; });
+      dft_tw<A, DIR, (n2 > 0)>(z[n2], [&](auto n1) { return tw[e * ((sn1 * n1 + sn2 * n2) % R)]; });
     });
-    dft<R, DIR, full_mask(R)>(x);
+    sfor<A>([&](auto k1) {
+      C v[B];
+      sfor<B>([&](auto n2) {
+        if constexpr (coprime) v[n2] = z[n2][k1];
+        else v[n2] = mul_c<R, n2 * k1, DIR>(z[n2][k1]);
+      });
+      dft<B, DIR, full_mask(B)>(v);
+      sfor<B>([&](auto k2) { x[(sk1 * k1 + sk2 * k2) % R] = v[k2]; });
+    });
   }
 }
 

@@ -17,7 +17,7 @@ double dft_ops(int R) {
   }
   int p = 2;
   while (R % p) ++p;
-  if (p == R) return (double)(p - 1) * (p + 4);
+  if (p == R) return p == 3 ? 12.0 : (double)(p - 1) * (p + 3);
   int A = p;
   while (R % (A * p) == 0) A *= p;
   if (A < R) return (R / A) * dft_ops(A) + A * dft_ops(R / A);
@@ -25,13 +25,14 @@ double dft_ops(int R) {
 }
 
 // ... behind twiddles: folded into the layers of a power of two, else four each
+// less two per first pair
 double dft_pre_ops(int R) {
   if ((R & (R - 1)) == 0) {
     double f = 0.0;
     for (int m = 2; m <= R; m *= 2) f += (double)(R / m) * 6.0 * (m / 2);
     return f;
   }
-  return dft_ops(R) + 4.0 * (R - 1);
+  return dft_ops(R) + 4.0 * (R - 1) - 2.0 * (R / 3);
 }
 
 }  // namespace

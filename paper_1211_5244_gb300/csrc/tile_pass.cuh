@@ -348,15 +348,20 @@ __global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_conv(const
 #pragma unroll
       for (int r = 0; r < R; ++r) x[r] = p[r * a.es];
       dft_pre<R, -1>(x, s.tw, e, a.Kl);
-      T el = T(0);
+      if (a.E != nullptr) {  // a solve without the energy saves its products
+        T el = T(0);
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const C u = mk(kk[r] * x[r].x, kk[r] * x[r].y);
-        el = mad(u.x, x[r].x, mad(u.y, x[r].y, el));  // K |rho^F|^2
-        x[r] = u;
+        for (int r = 0; r < R; ++r) {
+          const C u = mk(kk[r] * x[r].x, kk[r] * x[r].y);
+          el = mad(u.x, x[r].x, mad(u.y, x[r].y, el));  // K |rho^F|^2
+          x[r] = u;
+        }
+        const int k0 = a.w_tile ? line : pl;
+        en = mad(k0 == 0 || 2 * k0 == a.La0 ? T(1) : T(2), el, en);
+      } else {
+#pragma unroll
+        for (int r = 0; r < R; ++r) x[r] = mk(kk[r] * x[r].x, kk[r] * x[r].y);
       }
-      const int k0 = a.w_tile ? line : pl;
-      en = mad(k0 == 0 || 2 * k0 == a.La0 ? T(1) : T(2), el, en);
       dft<R, 1, full_mask(R)>(x);
 #pragma unroll
       for (int r = 0; r < R; ++r) p[r * a.es] = x[r];
