@@ -203,7 +203,7 @@ int check_solve_args(ps_plan p, const void* in, const void* out) {
   return PS_OK;
 }
 
-int run_solve(ps_plan p, const void* rho, void* V, double* E, cudaStream_t s) {
+int run_solve(ps_plan p, const void* rho, void* V, double* E, cudaStream_t s, VjpTerm* add = nullptr) {
   cudaError_t e;
   cudaEvent_t* ev = nullptr;
   if (p->profiling) {
@@ -216,9 +216,9 @@ int run_solve(ps_plan p, const void* rho, void* V, double* E, cudaStream_t s) {
     p->events_used += 6;
   }
   if (p->dtype == PS_F32)
-    e = launch_solve<float>(p, static_cast<const float*>(rho), static_cast<float*>(V), E, s, ev);
+    e = launch_solve<float>(p, static_cast<const float*>(rho), static_cast<float*>(V), E, s, ev, add);
   else
-    e = launch_solve<double>(p, static_cast<const double*>(rho), static_cast<double*>(V), E, s, ev);
+    e = launch_solve<double>(p, static_cast<const double*>(rho), static_cast<double*>(V), E, s, ev, add);
   if (e != cudaSuccess) return cuda_fail(e, "solve launch");
   return PS_OK;
 }
@@ -571,11 +571,12 @@ int ps_solve_vjp(ps_plan p, const void* vbar, const void* V, const double* gE_de
     return fail(PS_ERR_ARG, "pointers must be aligned to the element size");
   DeviceGuard g(p->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  VjpTerm term{V, gE_dev, false};
   if (vbar) {
-    int rc = run_solve(p, vbar, rhobar, nullptr, s);
+    int rc = run_solve(p, vbar, rhobar, nullptr, s, V ? &term : nullptr);
     if (rc != PS_OK) return rc;
   }
-  if (V) {
+  if (V && !term.fused) {
     cudaError_t e = p->dtype == PS_F32
         ? launch_vjp_axpy<float>(p, static_cast<float*>(rhobar), static_cast<const float*>(V), gE_dev,
                                  vbar != nullptr, s)

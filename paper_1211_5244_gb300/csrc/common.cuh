@@ -73,6 +73,14 @@ struct BlueArgs {
   const void* Bf;     // DFT_M of the conjugate chirp, divided by M
 };
 
+// The energy term h^3 gE V of a vector-Jacobian product, added by the last pass
+// to its outputs where its kernel does (`fused` tells)
+struct VjpTerm {
+  const void* V;
+  const double* gE;
+  bool fused;
+};
+
 // Arguments of the specialised FP32 pass kernels (strides in complex elements).
 struct FastArgs {
   int c;                  // valid kx columns (L1/2 + 1)
@@ -89,6 +97,9 @@ struct FastArgs {
   int rev;                // walk the z planes (y passes) or rows (x passes) from the last one:
                           // the previous pass wrote them last, so they are still in L2
   int nparts;             // inverse x pass: energy partials of the z pass, added by its first CTA
+  const float* addV;      // inverse x pass of a vector-Jacobian product: V += h3 gE addV
+  const double* gE;
+  double h3;
   const float2* tw1;      // fused x/y kernels: W_L1^k, k < L1 (set at launch)
 };
 
@@ -104,6 +115,7 @@ struct PassCfg {
                 // four-step convolution (0: Stockham stages)
   int fast;     // 1 if a compile-time specialised kernel runs this pass
   const void* fn;  // the specialised kernel
+  const void* fn_add;  // inverse x pass: the one that adds the energy term of a VJP
   dim3 grid, block;
   int cluster;  // CTAs per thread-block cluster (0: launched without clusters)
   int xrows;    // specialised x passes: rows per CTA
@@ -228,13 +240,14 @@ template <typename T>
 cudaError_t configure_passes(ps_plan_s* p);
 template <typename T>
 cudaError_t launch_solve(ps_plan_s* p, const T* rho, T* V, double* E, cudaStream_t s,
-                         cudaEvent_t* ev);
+                         cudaEvent_t* ev, VjpTerm* add = nullptr);
 template <typename T>
 cudaError_t launch_vjp_axpy(ps_plan_s* p, T* out, const T* V, const double* gE, bool accumulate,
                             cudaStream_t s);
 // passes_ord.cu: the solve for a processing order other than x, y, z
 template <typename T>
-cudaError_t launch_solve_ord(ps_plan_s* p, const T* rho, T* V, double* E, cudaStream_t s, cudaEvent_t* ev);
+cudaError_t launch_solve_ord(ps_plan_s* p, const T* rho, T* V, double* E, cudaStream_t s, cudaEvent_t* ev,
+                             VjpTerm* add);
 // energy partials (CTAs of the fused pass) of a plan in another order, and
 // the launch attributes of its kernels
 int ord_conv_ctas(const ps_plan_s* p);

@@ -148,7 +148,9 @@ __global__ void __launch_bounds__(TR*(P < Q ? P : Q), 4)
   }
 }
 
-template <int P, int Q, int TR, bool HALF, bool SH = false>
+// ADD: V += h3 gE addV, the energy term of a vector-Jacobian product, which took a pass
+// of its own over V and the result (192^3: 13 us)
+template <int P, int Q, int TR, bool HALF, bool SH = false, bool ADD = false>
 __global__ void __launch_bounds__(TR*(P < Q ? P : Q), SH ? 3 : 4)
     k_x_c2r(const void* src_v, void* dst_v, const float* twm_v, const float2* __restrict__ tw, FastArgs a,
             double* partials, unsigned*, double escale, double* E) {
@@ -235,6 +237,18 @@ __global__ void __launch_bounds__(TR*(P < Q ? P : Q), SH ? 3 : 4)
 #pragma unroll
     for (int k1 = 0; k1 < P; ++k1) y[k1] = ex[k1 * S::QP + b];
     rdft<P, 1, false>(y);
+    if constexpr (ADD) {
+      if (valid) {
+        const float f = (float)(a.h3 * __ldg(a.gE));
+        const float* w = a.addV + (long long)row * a.n1;
+#pragma unroll
+        for (int aa = 0; aa < NA; ++aa) {
+          const int m = b + Q * aa;
+          if (2 * m < a.n1) y[aa].x = fmaf(f, w[2 * m], y[aa].x);
+          if (2 * m + 1 < a.n1) y[aa].y = fmaf(f, w[2 * m + 1], y[aa].y);
+        }
+      }
+    }
     if (valid) {
 #pragma unroll
       for (int aa = 0; aa < NA; ++aa) {
@@ -258,9 +272,10 @@ static const void* pick_x(int kind, bool half) {
   if (kind == 0) return half ? (const void*)k_x_r2c<P, Q, TR, true> : (const void*)k_x_r2c<P, Q, TR, false>;
   // P = Q: the untangling by shuffles (three CTAs per SM; 44.4 against 45.7 us
   // at 256^3 for the shared-memory form)
-  if constexpr (P == Q)
-    return half ? (const void*)k_x_c2r<P, Q, TR, true, true> : (const void*)k_x_c2r<P, Q, TR, false, true>;
-  return half ? (const void*)k_x_c2r<P, Q, TR, true> : (const void*)k_x_c2r<P, Q, TR, false>;
+  constexpr bool SH = P == Q;
+  if (kind == 2)
+    return half ? (const void*)k_x_c2r<P, Q, TR, true, SH, true> : (const void*)k_x_c2r<P, Q, TR, false, SH, true>;
+  return half ? (const void*)k_x_c2r<P, Q, TR, true, SH> : (const void*)k_x_c2r<P, Q, TR, false, SH>;
 }
 
 const void* xline_kernel(int M, int kind, bool half, int* threads, int* rows, size_t* smem) {
@@ -357,6 +372,10 @@ cudaError_t configure_fast_f32(ps_plan_s* p) {
       if ((e = set(P1, f0, grid, threads, smem, base)) != cudaSuccess) return e;
       if ((e = set(P5, f1, grid, threads, smem, xinv)) != cudaSuccess) return e;
       p->cfg[P1].xrows = p->cfg[P5].xrows = rows;
+      p->cfg[P5].fn_add = xline_kernel(M, 2, half, &threads, &rows, &smem);
+      if (smem > 48 * 1024 && (e = cudaFuncSetAttribute(p->cfg[P5].fn_add, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                        (int)smem)) != cudaSuccess)
+        return e;
     }
   }
   // y passes (along b): nb <= Lb/2 (zero padding) or nb = Lb (periodic)
@@ -686,8 +705,8 @@ cudaError_t launch_fast_chunk(ps_plan_s* p, int pass, const void* rhoV, void* B,
 }
 
 cudaError_t launch_fast(ps_plan_s* p, int pass, const void* src, void* dst, double* E, double escale,
-                        cudaStream_t s) {
-  PassCfg& cf = p->cfg[pass];
+                        cudaStream_t s, VjpTerm* add) {
+  PassCfg cf = p->cfg[pass];
   const int axis = pass_axis(p, pass);
   // x passes get the twiddle matrix in the K slot
   const float* K = static_cast<const float*>((pass == P1 || pass == P5) ? p->twx : p->K);
@@ -696,6 +715,13 @@ cudaError_t launch_fast(ps_plan_s* p, int pass, const void* src, void* dst, doub
                    : ((pass == P2 && (p->ysoa & 1)) || (pass == P4 && (p->ysoa & 2))) ? p->tw4y : p->tw[axis];
   FastArgs fa = cf.fa;
   fa.nparts = z_pass_ctas(p);
+  if (pass == P5 && add != nullptr) {
+    cf.fn = cf.fn_add;
+    fa.addV = static_cast<const float*>(add->V);
+    fa.gE = add->gE;
+    fa.h3 = p->h * p->h * p->h;
+    add->fused = true;
+  }
   return launch_cfg(cf, fa, src, dst, K, tw, p->partials, p->counter, escale, E, s);
 }
 

@@ -55,7 +55,8 @@ using FastKernel = void (*)(const void*, void*, const float*, const float2*, Fas
 //   kind 0: forward (n nonzero inputs, L outputs), 1: inverse (L inputs,
 //   n outputs), 2: forward, K^F multiply, inverse; half: n = L/2 (else n = L)
 const void* strided_kernel(int L, int kind, bool half, int* threads, size_t* smem, int* tk);
-// Returns the kernel for an x pass (real length 2M): kind 0 R2C, 1 C2R.
+// Returns the kernel for an x pass (real length 2M): kind 0 R2C, 1 C2R, 2 C2R that adds the
+// energy term of a vector-Jacobian product.
 const void* xline_kernel(int M, int kind, bool half, int* threads, int* rows, size_t* smem);
 
 // The persistent packed y-pass kernels (L2 = 512), or nullptr.
@@ -88,8 +89,9 @@ cudaError_t configure_fast_f32(ps_plan_s* p);
 
 // Launches pass `pass` with its specialised kernel. E (or NULL): the z pass stores
 // its energy partials, the inverse x pass (and the inverse fused x/y kernel) adds them.
+// add (or NULL): the energy term of a VJP, taken by the inverse x pass.
 cudaError_t launch_fast(ps_plan_s* p, int pass, const void* src, void* dst, double* E, double escale,
-                        cudaStream_t s);
+                        cudaStream_t s, VjpTerm* add = nullptr);
 // Launches the fused forward (kind 0: rho -> B) or inverse (kind 1: B -> V) x/y kernel.
 cudaError_t launch_xy(ps_plan_s* p, int kind, const void* src, void* dst, double* E, double escale, cudaStream_t s);
 // Launches x pass P1 / P5 or y pass P2 / P4 on the z planes z0 .. z0 + nz - 1:

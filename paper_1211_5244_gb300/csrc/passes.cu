@@ -615,9 +615,9 @@ cudaError_t configure_passes(ps_plan_s* p) {
 
 template <typename T>
 cudaError_t launch_solve(ps_plan_s* p, const T* rho, T* V, double* E, cudaStream_t s,
-                         cudaEvent_t* ev) {
+                         cudaEvent_t* ev, VjpTerm* add) {
   using C = cpx<T>;
-  if (!canonical_order(p) && !p->fastord) return launch_solve_ord<T>(p, rho, V, E, s, ev);
+  if (!canonical_order(p) && !p->fastord) return launch_solve_ord<T>(p, rho, V, E, s, ev, add);
   C* A = static_cast<C*>(p->A);
   C* B = static_cast<C*>(p->B);
   const C* tw0 = static_cast<const C*>(p->tw[0]);
@@ -723,9 +723,9 @@ cudaError_t launch_solve(ps_plan_s* p, const T* rho, T* V, double* E, cudaStream
   if (xyf) {
     // done by the fused kernel above
   } else if (p->cfg[P5].fast && a8) {
-    if ((e = launch_fast(p, P5, A, V, Ez, escale, s)) != cudaSuccess) return e;
+    if ((e = launch_fast(p, P5, A, V, Ez, escale, s, add)) != cudaSuccess) return e;
   } else if (p->tile[P5].on) {
-    if ((e = launch_tile(p, P5, A, V, Ez, s)) != cudaSuccess) return e;
+    if ((e = launch_tile(p, P5, A, V, Ez, s, add)) != cudaSuccess) return e;
   } else {
     GenArgs a = gen_args<T>(p, P5);
     const int rpc = (p->L[0] % 2 == 0) ? a.tk : 2 * a.tk;  // odd L1: two real rows per line
@@ -759,8 +759,8 @@ template cudaError_t launch_x_pass<double>(ps_plan_s*, int, const void*, void*, 
 template cudaError_t configure_passes<float>(ps_plan_s*);
 template cudaError_t configure_passes<double>(ps_plan_s*);
 template cudaError_t launch_solve<float>(ps_plan_s*, const float*, float*, double*, cudaStream_t,
-                                         cudaEvent_t*);
+                                         cudaEvent_t*, VjpTerm*);
 template cudaError_t launch_solve<double>(ps_plan_s*, const double*, double*, double*, cudaStream_t,
-                                          cudaEvent_t*);
+                                          cudaEvent_t*, VjpTerm*);
 
 }  // namespace ps

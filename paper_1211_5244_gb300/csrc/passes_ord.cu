@@ -345,7 +345,8 @@ int ord_conv_ctas(const ps_plan_s* p) {
 }
 
 template <typename T>
-cudaError_t launch_solve_ord(ps_plan_s* p, const T* rho, T* V, double* E, cudaStream_t s, cudaEvent_t* ev) {
+cudaError_t launch_solve_ord(ps_plan_s* p, const T* rho, T* V, double* E, cudaStream_t s, cudaEvent_t* ev,
+                             VjpTerm* add) {
   using C = cpx<T>;
   C* A = static_cast<C*>(p->A);
   C* B = static_cast<C*>(p->B);
@@ -386,7 +387,7 @@ cudaError_t launch_solve_ord(ps_plan_s* p, const T* rho, T* V, double* E, cudaSt
   }
   if (ev) cudaEventRecord(ev[4], s);
   if (p->tile[P5].on) {
-    if ((e = launch_tile(p, P5, A, V, E, s)) != cudaSuccess) return e;
+    if ((e = launch_tile(p, P5, A, V, E, s, add)) != cudaSuccess) return e;
   } else if (xfirst) {
     if ((e = launch_x_pass<T>(p, P5, A, V, E, s)) != cudaSuccess) return e;
   } else {
@@ -414,9 +415,11 @@ cudaError_t configure_ord(const ps_plan_s*) {
   return cudaFuncSetAttribute(ord_c2r<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, budget);
 }
 
-template cudaError_t launch_solve_ord<float>(ps_plan_s*, const float*, float*, double*, cudaStream_t, cudaEvent_t*);
+template cudaError_t launch_solve_ord<float>(ps_plan_s*, const float*, float*, double*, cudaStream_t, cudaEvent_t*,
+                                             VjpTerm*);
 template cudaError_t launch_solve_ord<double>(ps_plan_s*, const double*, double*, double*, cudaStream_t,
-                                              cudaEvent_t*);
+                                              cudaEvent_t*,
+                                              VjpTerm*);
 template cudaError_t configure_ord<float>(const ps_plan_s*);
 template cudaError_t configure_ord<double>(const ps_plan_s*);
 

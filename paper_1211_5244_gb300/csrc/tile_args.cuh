@@ -8,6 +8,8 @@ struct ps_plan_s;
 
 namespace ps {
 
+struct VjpTerm;
+
 // A line of length N = Ra Rm Rl (Rm = 1 for two steps): digits n = n1 NRa + n2 Rl
 // + n3 of the input index, k = k1 + Ra k2 + Ra Rm k3 of the output index.
 struct TileArgs {
@@ -41,6 +43,10 @@ struct TileArgs {
   // energy: partials of the fused pass, added by the last pass's first CTA
   double* partials;
   int nparts;
+  // last pass of a vector-Jacobian product: outputs += h3 gE addV
+  const void* addV;
+  const double* gE;
+  double h3;
   int shift;  // 1: the first CTA in x adds the partials and has no lines
   double escale;
   double* E;
@@ -87,6 +93,7 @@ template <typename T> const void* tile_blue_kernel(int pass, bool pair);
 // Fills p->tile[pass] for the passes that run here (before npart is taken).
 template <typename T> cudaError_t configure_tile(ps_plan_s* p);
 // Launches pass `pass`; src and dst as in launch_solve.
-cudaError_t launch_tile(ps_plan_s* p, int pass, const void* src, void* dst, double* E, cudaStream_t s);
+cudaError_t launch_tile(ps_plan_s* p, int pass, const void* src, void* dst, double* E, cudaStream_t s,
+                        VjpTerm* add = nullptr);
 
 }  // namespace ps

@@ -325,7 +325,8 @@ cudaError_t configure_tile(ps_plan_s* p) {
 template cudaError_t configure_tile<float>(ps_plan_s*);
 template cudaError_t configure_tile<double>(ps_plan_s*);
 
-cudaError_t launch_tile(ps_plan_s* p, int pass, const void* src, void* dst, double* E, cudaStream_t s) {
+cudaError_t launch_tile(ps_plan_s* p, int pass, const void* src, void* dst, double* E, cudaStream_t s,
+                        VjpTerm* add) {
   const TileLaunch& tl = p->tile[pass];
   TileArgs a = tl.a;
   const int al = pass_axis(p, pass);
@@ -340,6 +341,12 @@ cudaError_t launch_tile(ps_plan_s* p, int pass, const void* src, void* dst, doub
   a.nparts = z_pass_ctas(p);
   a.escale = 0.5 * p->h * p->h * p->h;
   a.E = E;
+  if (pass == P5 && add != nullptr) {
+    a.addV = add->V;
+    a.gE = add->gE;
+    a.h3 = p->h * p->h * p->h;
+    add->fused = true;
+  }
   if (a.vec) {
     const void* r = pass == P1 ? src : dst;
     a.vec = reinterpret_cast<uintptr_t>(r) % (2 * p->esz) == 0;

@@ -412,12 +412,19 @@ __device__ __forceinline__ bool energy_cta(const TileArgs& a) {
 template <typename T, bool PAIR>
 struct RealLine {
   T* p0;
+  const T* add;  // the energy term's V at the line, and its factor
+  T fac;
   bool ok, two;
   __device__ __forceinline__ RealLine(const TileArgs& a, const void* base, long long sp, long long st, int t) {
     int line, pl;
     ok = line_of(a, t, &line, &pl);
     p0 = const_cast<T*>(static_cast<const T*>(base)) + (pl * sp + line * st);
     two = PAIR && 2 * line + 1 < a.nreal;
+    add = nullptr;
+    if (a.addV != nullptr) {
+      add = static_cast<const T*>(a.addV) + (pl * sp + line * st);
+      fac = (T)(a.h3 * __ldg(a.gE));
+    }
   }
   __device__ __forceinline__ cpx<T> load(const TileArgs& a, int e) const {
     cpx<T> v = mk(T(0), T(0));
@@ -433,6 +440,11 @@ struct RealLine {
     if (!ok || e >= a.nout) return;
     T* p = p0 + (long long)e * a.se_out;
     const bool im = PAIR ? two : 2 * e + 1 < a.nreal;
+    if (add != nullptr) {
+      const T* q = add + (long long)e * a.se_out;
+      v.x = mad(fac, q[0], v.x);
+      if (im) v.y = mad(fac, q[a.im_off], v.y);
+    }
     if (a.vec && im) {
       *reinterpret_cast<cpx<T>*>(p) = v;
     } else {
