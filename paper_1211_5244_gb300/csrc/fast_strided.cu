@@ -242,12 +242,10 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
   constexpr int NB = Q / T;
   constexpr int NK = P / T;
   constexpr int NA = HALF ? P / 2 : P;
-  constexpr int ROWS = NA * Q;      // input rows of a line
   constexpr int KROWS = L / 2 + 1;  // rows of the K^F octant
   constexpr int RG = TK * 8 < 128 ? P : 0;  // exchange rows per padded group (0: no padding)
   static_assert(RG == 0 || (P == RG && Q == RG), "padded exchange: P = Q = rows per group");
   constexpr int PP = RG ? P + 1 : P;         // row pitch of b in the exchange (rows b * PP + k1)
-  constexpr int QQ = RG ? Q + 1 : Q;         // row pitch of aa for the input rows b + Q aa
   constexpr int LP = RG ? L + L / RG : L;    // exchange rows including the padding
   extern __shared__ float2 sh[];    // exchange [LP][TK]; the K^F slice [KROWS][TK] floats; W_L^i, i < L
   float* const kstage = reinterpret_cast<float*>(sh + LP * TK);
@@ -262,14 +260,16 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
 
   constexpr int NT = TK * T;
   constexpr int IPR = TK / 2;  // 16-byte pieces per input row
-  constexpr int ISTEP = NT / IPR;
-  static_assert(NT % IPR == 0 && ROWS % ISTEP == 0, "input copy shape");
-  static_assert(RG == 0 || ISTEP % RG == 0, "padded input copy shape");
-  constexpr int ISTEPP = RG ? ISTEP + ISTEP / RG : ISTEP;  // exchange rows per sweep, padding included
-  const int irow0 = threadIdx.x / IPR;
+  // the rows b + Q aa of column b land in the exchange rows (b, aa), which only the
+  // threads of column b (j = b) read and then write, copied by their own warp two aa at a time:
+  // the inputs need no barrier of the CTA
+  static_assert(NB == 1 && NA % 2 == 0 && 32 % TK == 0, "input copy shape");
+  constexpr int GPW = 32 / TK;  // columns per warp
+  const int lj = (threadIdx.x / 32) * GPW + (threadIdx.x % 32) / IPR % GPW, lh = (threadIdx.x % 32) / (IPR * GPW);
+  const int irow0 = lj + Q * lh;
   const long long igoff = (long long)irow0 * es + 2 * (threadIdx.x % IPR);
-  const long long igstep = (long long)ISTEP * es;
-  float2* const is0 = sh + (RG ? irow0 + irow0 / RG : irow0) * TK + 2 * (threadIdx.x % IPR);
+  const long long igstep = (long long)(2 * Q) * es;
+  float2* const is0 = sh + (lj * PP + lh) * TK + 2 * (threadIdx.x % IPR);
   const int ivalid = a.nl - irow0;
   constexpr int KPR = TK / 4;  // 16-byte pieces per K^F row
   constexpr int KSTEP = NT / KPR;
@@ -292,11 +292,11 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
     const float2* src0 = base + paired_ky(yi, a.L2) * a.src_plane + (a.kt0 + kt) * TK;
     const float2* src = src0 + igoff;
 #pragma unroll
-    for (int i = 0; i < ROWS / ISTEP; ++i) {
-      if (ISTEP * i < ivalid)
-        cp_async16(is0 + i * ISTEPP * TK, src);
+    for (int i = 0; i < NA / 2; ++i) {
+      if (2 * Q * i < ivalid)
+        cp_async16(is0 + i * 2 * TK, src);
       else  // beyond the physical z rows: zeros (nothing is read)
-        cp_async16_zero(is0 + i * ISTEPP * TK, src0);
+        cp_async16_zero(is0 + i * 2 * TK, src0);
       src += igstep;
     }
   };
@@ -320,6 +320,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
   pdl_wait();
   if (tile < ntiles) issue_input(kt, yi);
   cp_async_commit();
+  __syncthreads();  // the twiddle table
   for (; tile < ntiles; tile += gridDim.x) {
     const int next = tile + gridDim.x;
     const int kx = (a.kt0 + kt) * TK + t;
@@ -327,7 +328,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
     const int ky = paired_ky(yi, a.L2);
     float2* line = base + ky * a.src_plane + kx;
     cp_async_wait_all();
-    __syncthreads();  // this tile's input rows and K^F slice have landed
+    __syncwarp();  // the warp's input rows have landed; the K^F slice is read after the next barrier
 
     float2 y[NB][P];
 #pragma unroll
@@ -336,10 +337,10 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
 #pragma unroll
       for (int aa = 0; aa < P; ++aa) {
         y[u][aa] = make_float2(0.f, 0.f);
-        if (aa < NA && valid) y[u][aa] = sh[(b + QQ * aa) * TK + t];
+        if (aa < NA && valid) y[u][aa] = sh[(b * PP + aa) * TK + t];
       }
     }
-    __syncthreads();  // inputs read: the space becomes the exchange
+    __syncwarp();  // inputs read: the warp's rows become the exchange
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
       const int b = j + T * u;
@@ -385,7 +386,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
 #pragma unroll
       for (int k1 = 0; k1 < P; ++k1) y[u][k1] = sh[(b * PP + k1) * TK + t];
     }
-    __syncthreads();  // the exchange has been read: the next tile's rows may land in it
+    __syncwarp();  // the warp has read its rows: the next tile's may land in them
     if (next < ntiles) issue_input(nkt, nyi);
     cp_async_commit();
 #pragma unroll
@@ -449,16 +450,14 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
     k_ypipe(const void* src_v, void* dst_v, const float*, const float2* __restrict__ tw, FastArgs a, double*,
             unsigned*, double, double*) {
   pdl_wait();
-  constexpr int L = P * Q;
   constexpr int T = P < Q ? P : Q;
   constexpr int NB = Q / T;
   constexpr int NK = P / T;
   constexpr int NA = HALF ? P / 2 : P;
-  constexpr int ROWS = KIND == 0 ? NA * Q : L;  // input rows of a line
   constexpr int RG = TK * 8 < 128 ? P : 0;      // exchange rows per padded group (0: no padding)
   static_assert(RG == 0 || (P == RG && Q == RG), "padded exchange: P = Q = rows per group");
   constexpr int PP = RG ? P + 1 : P;             // row pitch of b in the exchange (rows b * PP + k1)
-  extern __shared__ float2 sh[];               // inputs [ROWS][TK]; later, in the same space, the exchange [L + L / RG][TK]
+  extern __shared__ float2 sh[];               // the exchange [L + L / RG][TK]; the inputs land in its rows
   const float2* src = static_cast<const float2*>(src_v);
   float2* dst = static_cast<float2*>(dst_v);
   const int t = threadIdx.x % TK;
@@ -466,28 +465,45 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
   const int ntk = a.ntk_loc;  // kx tiles a.kt0 .. a.kt0 + ntk - 1
   const int ntiles = ntk * (int)a.nrows;  // nrows = number of z planes here
 
-  // the input copy: ROWS rows of TK float2 in 16-byte pieces, a fixed number
-  // of sweeps of the CTA, per-thread offsets computed once
+  // the input copy: rows of TK float2 in 16-byte pieces, per-thread offsets
+  // computed once
   constexpr int NT = TK * T;
   constexpr int IPR = TK / 2;
-  constexpr int ISTEP = NT / IPR;
-  static_assert(NT % IPR == 0 && ROWS % ISTEP == 0, "input copy shape");
-  const int irow0 = threadIdx.x / IPR;
+  // the rows land where only the threads that read them write next, copied by their
+  // own warp (no CTA barrier for the inputs): forward, row b + Q aa in the exchange row (b, aa), b = j + T u;
+  // inverse, row k1 + P k2 in (k2, k1), k1 = j + T v
+  static_assert(NA % 2 == 0 && Q % 2 == 0 && 32 % TK == 0 && NT % 32 == 0, "input copy shape");
+  constexpr int GPW = 32 / TK;  // thread groups j per warp
+  const int lj = (threadIdx.x / 32) * GPW + (threadIdx.x % 32) / IPR % GPW, lh = (threadIdx.x % 32) / (IPR * GPW);
+  const int irow0 = lj + (KIND == 0 ? Q : P) * lh;
   const long long igoff = (long long)irow0 * a.src_elem + 2 * (threadIdx.x % IPR);
-  const long long igstep = (long long)ISTEP * a.src_elem;
-  float2* const is0 = sh + irow0 * TK + 2 * (threadIdx.x % IPR);
-  const int ivalid = a.nl - irow0;  // sweep i copies a physical row iff ISTEP * i < ivalid
+  float2* const is0 = sh + (KIND == 0 ? lj * PP + lh : lh * PP + lj) * TK + 2 * (threadIdx.x % IPR);
+  const int ivalid = a.nl - irow0;  // forward: a copy is of a physical row iff 2 Q i + T u < ivalid
   auto plane = [&](int zi) { return a.rev ? (int)a.nrows - 1 - zi : zi; };
   auto prefetch = [&](int kt, int zi) {
     const float2* sp0 = src + (long long)plane(zi) * a.src_plane + (a.kt0 + kt) * TK;
     const float2* sp = sp0 + igoff;
+    if constexpr (KIND == 0) {
+      const long long ustep = (long long)T * a.src_elem, step = (long long)(2 * Q) * a.src_elem;
 #pragma unroll
-    for (int i = 0; i < ROWS / ISTEP; ++i) {
-      if (KIND == 1 || ISTEP * i < ivalid)
-        cp_async16(is0 + i * ISTEP * TK, sp);
-      else  // beyond the physical rows of the plane: zeros
-        cp_async16_zero(is0 + i * ISTEP * TK, sp0);
-      sp += igstep;
+      for (int i = 0; i < NA / 2; ++i) {
+#pragma unroll
+        for (int u = 0; u < NB; ++u) {
+          if (2 * Q * i + T * u < ivalid)
+            cp_async16(is0 + (T * u * PP + i * 2) * TK, sp + u * ustep);
+          else  // beyond the physical rows of the plane: zeros
+            cp_async16_zero(is0 + (T * u * PP + i * 2) * TK, sp0);
+        }
+        sp += step;
+      }
+    } else {
+      const long long vstep = (long long)T * a.src_elem, step = (long long)(2 * P) * a.src_elem;
+#pragma unroll
+      for (int i = 0; i < Q / 2; ++i) {
+#pragma unroll
+        for (int v = 0; v < NK; ++v) cp_async16(is0 + (i * 2 * PP + T * v) * TK, sp + v * vstep);
+        sp += step;
+      }
     }
   };
   // tile = kt + ntk * zi (kx tile fastest); the CTA steps by gridDim.x tiles
@@ -513,7 +529,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
     const bool valid = kx < a.c;
     float2* d = dst + (long long)plane(zi) * a.dst_plane + kx;
     cp_async_wait_all();
-    __syncthreads();  // the tile's rows have landed
+    __syncwarp();  // the warp's rows have landed
     float2 X[NK][Q];
     if constexpr (KIND == 0) {
       float2 y[NB][P];
@@ -523,10 +539,10 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
 #pragma unroll
         for (int aa = 0; aa < P; ++aa) {
           y[u][aa] = make_float2(0.f, 0.f);
-          if (aa < NA && valid) y[u][aa] = sh[(b + Q * aa) * TK + t];
+          if (aa < NA && valid) y[u][aa] = sh[(b * PP + aa) * TK + t];
         }
       }
-      __syncthreads();  // inputs read: the tile becomes the exchange
+      __syncwarp();  // inputs read: the warp's rows become the exchange
 #pragma unroll
       for (int u = 0; u < NB; ++u) {
         const int b = j + T * u;
@@ -559,9 +575,9 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
         const int k1 = j + T * v;
 #pragma unroll
         for (int k2 = 0; k2 < Q; ++k2)
-          X[v][k2] = valid ? sh[(k1 + P * k2) * TK + t] : make_float2(0.f, 0.f);
+          X[v][k2] = valid ? sh[(k2 * PP + k1) * TK + t] : make_float2(0.f, 0.f);
       }
-      __syncthreads();  // inputs read: the tile becomes the exchange
+      __syncwarp();  // inputs read: the warp's rows become the exchange
 #pragma unroll
       for (int v = 0; v < NK; ++v) {
         const int k1 = j + T * v;
