@@ -11,7 +11,8 @@
 // unnormalised length-L1 inverse at even (real part) and odd (imaginary part)
 // positions. T lanes own one row (contiguous 8-byte elements), so loads and
 // stores are coalesced along the row. With zero padding (n1 = M), inputs
-// z[m] with m >= M/2 are zero and outputs there are never formed.
+// z[m] with m >= M/2 are zero and outputs there are never formed. The T lanes of a row
+// (4, 8 or 16) sit in one warp, so the exchanges need the warp's barriers only.
 #include <algorithm>
 #include <cstdlib>
 #include <cstring>
@@ -87,7 +88,7 @@ __global__ void __launch_bounds__(TR*(P < Q ? P : Q), 4)
 #pragma unroll
     for (int k1 = 0; k1 < P; ++k1) ex[k1 * S::QP + b] = y[k1];
   }
-  __syncthreads();
+  __syncwarp();
   float2 x[NK][Q];
 #pragma unroll
   for (int v = 0; v < NK; ++v) {
@@ -122,7 +123,7 @@ __global__ void __launch_bounds__(TR*(P < Q ? P : Q), 4)
     }
     return;
   }
-  __syncthreads();  // the exchange has been read: its space takes the row spectrum
+  __syncwarp();  // the exchange has been read: its space takes the row spectrum
 #pragma unroll
   for (int v = 0; v < NK; ++v) {
     const int k1 = j + T * v;
@@ -130,7 +131,7 @@ __global__ void __launch_bounds__(TR*(P < Q ? P : Q), 4)
 #pragma unroll
     for (int k2 = 0; k2 < Q; ++k2) zr[k1 + P * k2] = x[v][k2];
   }
-  __syncthreads();
+  __syncwarp();
   if (!valid) return;
   // outputs k and M - k from the same pair Z[k], Z[M - k]: E[M-k] = conj E[k],
   // O[M-k] = conj O[k] and W_L1^{M-k} = -conj W_L1^k, so X[M-k] = conj(E[k] - W^k O[k])
@@ -202,7 +203,7 @@ __global__ void __launch_bounds__(TR*(P < Q ? P : Q), SH ? 3 : 4)
     for (int i = 0; i < M / T; ++i) xr[j + T * i] = xin[i];
     if (j == 0) xr[M] = xny;
   }
-  __syncthreads();
+  __syncwarp();
 #pragma unroll
   for (int v = 0; v < NK; ++v) {
     const int k1 = j + T * v;
@@ -215,7 +216,7 @@ __global__ void __launch_bounds__(TR*(P < Q ? P : Q), SH ? 3 : 4)
       x[v][k2] = make_float2(e.x - o.y, e.y + o.x);
     }
   }
-  __syncthreads();  // the row spectrum has been read: its space takes the exchange
+  __syncwarp();  // the row spectrum has been read: its space takes the exchange
   }
 
 #pragma unroll
@@ -229,7 +230,7 @@ __global__ void __launch_bounds__(TR*(P < Q ? P : Q), SH ? 3 : 4)
     for (int b2 = 0; b2 < Q / 2; ++b2)
       w4[b2] = make_float4(x[v][2 * b2].x, x[v][2 * b2].y, x[v][2 * b2 + 1].x, x[v][2 * b2 + 1].y);
   }
-  __syncthreads();
+  __syncwarp();
 #pragma unroll
   for (int u = 0; u < NB; ++u) {
     const int b = j + T * u;
