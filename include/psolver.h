@@ -168,7 +168,7 @@ int ps_plan_set_lengths(ps_plan plan, int L1, int L2, int L3);
  * rule: periodic axes first (their transforms run before any zero padding
  * exists), free axes last, so that wire BCs do 7/12 and surface BCs 2/3 of a
  * full padded 3D FFT's 1D transforms for any assignment of the axes. Orders
- * other than x, y, z run the generic kernels along strided axes (the
+ * other than x, y, z run the tile kernels along strided axes (the
  * specialised FP32 kernels, the fused x/y passes and the tensor-core z pass
  * need x first); every order gives the same result up to rounding. No
  * transpose: the passes index the x-fastest arrays through strides.
@@ -184,8 +184,8 @@ int ps_plan_set_order(ps_plan plan, int a0, int a1, int a2);
  * >= 2n - 1 with register-resident FP32 kernels (a power of two, 96, 192 or
  * 384). Then, at the fastest lengths, each schedule
  * choice that applies to the plan is timed in turn and kept if faster: the
- * lines per tile of the generic passes, their radix split (radix 8 first or
- * radix 4 only), both again per physical axis, the lines per tile of the persistent packed z kernel, the y
+ * lines per tile of the passes without a specialised kernel, their radix choice
+ * (tile kernels or Stockham stages), both again per physical axis, the lines per tile of the persistent packed z kernel, the y
  * kernel form (packed persistent, unpacked persistent, non-persistent), the
  * fused x/y passes (see ps_plan_info.fused), the chunks of the x and y passes
  * and, for a plan whose order is not x first, the x-first order. One trial plan per candidate
@@ -209,7 +209,9 @@ int ps_plan_set_math(ps_plan plan, int math_mode);
  * up to rounding; a choice that does not apply to the plan's shapes is
  * ignored. 0 keeps a field's default.
  *   tile    most lines per tile of the generic passes: 0, 1, 2, 4, 8, 16 or 32
- *   radix   generic Stockham stages: 0 radix 8 first, 1 radix 4 and 2 only
+ *   radix   passes without a specialised kernel: 0 the tile kernels (register
+ *           DFT steps), with Stockham stages of radix 8 first where they have no
+ *           form for the length; 1 Stockham stages of radix 4 and 2 only
  *   ztk     lines per tile of the persistent packed z kernel: 0, 8 or 16
  *   ykind   y kernels: 0 default, 1 unpacked persistent, 2 non-persistent
  *   xy      1: fused x/y passes where the shapes have them (ps_plan_info.fused)
@@ -226,8 +228,7 @@ int ps_plan_set_schedule(ps_plan plan, int tile, int radix, int ztk, int ykind, 
  * them axis by axis). Same results up to rounding.
  *   tile    most lines per tile of the generic passes along the axis: 0 (the
  *           plan-wide tile), 1, 2, 4, 8, 16 or 32
- *   radix   their Stockham stages: -1 (the plan-wide radix), 0 radix 8 first,
- *           1 radix 4 and 2 only
+ *   radix   as in ps_plan_set_schedule; -1: the plan-wide radix
  * Errors: PS_ERR_ARG (plan NULL or built, axis or a value out of range).
  */
 int ps_plan_set_axis_schedule(ps_plan plan, int axis, int tile, int radix);

@@ -261,6 +261,8 @@ int gen_rows(const ps_plan_s* p, int pass);
 // that processes x first, on A with pitch ld1
 template <typename T>
 cudaError_t launch_x_pass(ps_plan_s* p, int pass, const void* src, void* dst, double* E, cudaStream_t s);
+// programmatic dependent launches (PS_PDL=0: off)
+bool pdl_launches();
 cudaError_t build_twiddles(ps_plan_s* p, cudaStream_t s);
 // batch.cu: the batch as one cached CUDA graph of concurrent per-problem chains
 cudaError_t batch_solve_graph(int count, ps_plan_s* const* plans, const void* const* rho, void* const* V,

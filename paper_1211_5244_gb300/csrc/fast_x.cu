@@ -609,6 +609,14 @@ cudaError_t configure_fast_f32(ps_plan_s* p) {
   return cudaSuccess;
 }
 
+bool pdl_launches() {
+  static const bool pdl = [] {
+    const char* v = getenv("PS_PDL");
+    return !(v && atoi(v) == 0);
+  }();
+  return pdl;
+}
+
 namespace {
 
 // One launch of a specialised kernel: programmatic stream serialisation
@@ -620,10 +628,6 @@ cudaError_t launch_cfg(const PassCfg& cf, const FastArgs& fa, const void* src, v
   FastArgs a = fa;
   void* args[] = {(void*)&src, (void*)&dst, (void*)&K, (void*)&tw, (void*)&a,
                   (void*)&partials, (void*)&counter, (void*)&escale, (void*)&E};
-  static const bool pdl = [] {
-    const char* v = getenv("PS_PDL");
-    return !(v && atoi(v) == 0);
-  }();
   cudaLaunchConfig_t lc = {};
   lc.gridDim = cf.grid;
   lc.blockDim = cf.block;
@@ -631,7 +635,7 @@ cudaError_t launch_cfg(const PassCfg& cf, const FastArgs& fa, const void* src, v
   lc.stream = s;
   cudaLaunchAttribute attr[3];
   int na = 0;
-  if (pdl) {
+  if (pdl_launches()) {
     attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[na].val.programmaticStreamSerializationAllowed = 1;
     ++na;

@@ -365,7 +365,7 @@ cudaError_t launch_tile(ps_plan_s* p, int pass, const void* src, void* dst, doub
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   lc.attrs = attr;
-  lc.numAttrs = 1;
+  lc.numAttrs = pdl_launches() ? 1 : 0;
   return cudaLaunchKernelExC(&lc, tl.fn, args);
 }
 

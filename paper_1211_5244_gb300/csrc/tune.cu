@@ -11,8 +11,8 @@
 //   tile    lines per tile of the generic passes (32 / 16 / 8 / 4 in FP32,
 //           16 / 8 / 4 / 2 in FP64: wider tiles give each thread more
 //           butterflies per stage, narrower ones more CTAs per line set)
-//   radix   radix split of the generic Stockham stages (radix 8 first, or
-//           radix 4 and 2 only)
+//   radix   the tile kernels (Stockham stages of radix 8 first where they have
+//           no form for the length), or Stockham stages of radix 4 and 2 only
 //   tile and radix again per axis: for the generic passes along each
 //           physical axis on its own (ps_plan_set_axis_schedule)
 //   ztk     lines per tile of the persistent packed z kernel (8 or 16)
