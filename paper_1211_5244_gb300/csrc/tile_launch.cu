@@ -116,6 +116,13 @@ void tile_axes(int al, int* at, int* ap) {
 // thread per butterfly; L = 240: 16.3 us against 18.3 with 32 lines; L = 320:
 // 23.1 against 24.6).
 //
+// A fused z pass of few CTAs takes more threads per CTA: below 256 threads per SM
+// the chip is idle for want of warps, and the steps of one tile are its time. The
+// most threads whose last round of butterflies is not emptier by more than a tenth
+// (90 x 75 x 110 ppf, L3 = 220, 450 CTAs: 64 -> 192 threads, solve 32.7 -> 28.5 us).
+// With the line at 768 threads per SM a batch of 32 such problems, which fills the
+// chip, goes from 865 to 894 us; the other passes gain nothing from more threads.
+//
 // In FP64 a warp instruction holds the pipe as long with one lane as with 32: the
 // tile is the width with the fewest operations per SM, counting whole warps and
 // whole tiles, and the threads those that split the steps' butterflies most evenly
@@ -123,7 +130,8 @@ void tile_axes(int al, int* at, int* ap) {
 // rows count 5% more.
 // At most 72 KB, three CTAs per SM, else the widest tile that fits one.
 struct TileShape { int tk, threads; };
-TileShape pick_tile(const TileArgs& a, const TileRadix& r, int row, long long lines, int want, size_t esz, int sms) {
+TileShape pick_tile(const TileArgs& a, const TileRadix& r, int row, long long lines, int want, size_t esz, int sms,
+                    bool conv) {
   const size_t csz = 2 * esz;
   const bool f32 = esz == 4;
   const int nb[3] = {a.NRa, a.Kl, r.Rm > 1 ? r.Ra * r.Rl : 0};
@@ -151,11 +159,21 @@ TileShape pick_tile(const TileArgs& a, const TileRadix& r, int row, long long li
   const int most = tk * std::max(nb[0], std::max(nb[1], nb[2]));
   const int cap = (std::min(most, 256) + 31) / 32 * 32;
   int threads = std::min(cap, std::max(64, (a.N <= 288 ? 8 : 16) * tk));
+  auto rounds = [&](int th) {  // thread-operations of a CTA, idle threads of the last rounds counted
+    double w = 0.0;
+    for (int k = 0; k < 3; ++k) w += (double)((tk * nb[k] + th - 1) / th * th) * ops[k];
+    return w;
+  };
+  const long long ctas = (lines + tk - 1) / tk;
+  if (f32 && conv && ctas * threads < 256LL * sms) {
+    const int base = threads;
+    for (int th = base + 32; th <= cap; th += 32)
+      if (rounds(th) <= 1.1 * rounds(base)) threads = th;
+  }
   if (!f32) {
     double best = -1.0;
     for (int th = std::min(cap, 128); th <= cap; th += 32) {
-      double w = 0.0;
-      for (int k = 0; k < 3; ++k) w += (tk * nb[k] + th - 1) / th * th * ops[k];
+      const double w = rounds(th);
       if (best < 0.0 || w < best) {
         best = w;
         threads = th;
@@ -276,7 +294,7 @@ cudaError_t configure_pass(ps_plan_s* p, int pass, int sms) {
     }
   }
   const long long lines = (long long)a.ntl * a.npl;
-  const TileShape sh = pick_tile(a, r, row, lines, axis_tile(p, al), sizeof(T), sms);
+  const TileShape sh = pick_tile(a, r, row, lines, axis_tile(p, al), sizeof(T), sms, pass == P3);
   const int tk = sh.tk;
   if (tk == 0) return cudaSuccess;
   a.tk = tk;
