@@ -252,9 +252,15 @@ __device__ __forceinline__ void step_inv_first(const TileArgs& a, const Tile<C>&
   });
 }
 
+// Resident CTAs (of 256 threads) per SM asked of the compiler. The FP32 passes are
+// bound by latency, so more warps pay where the radices still fit their registers:
+// the real and the Bluestein passes take one CTA more (64 registers for class 1; 32
+// uneven problems 860 -> 834 us). The fused pass spills there (128^3 ffp 59.3 ->
+// 64.7 us), and the line pass loses by it (100 x 90 x 110 free 62.0 -> 63.0 us).
 template <typename T, int CLS>
-struct Bounds {  // resident CTAs per SM asked of the compiler
+struct Bounds {
   static constexpr int per_sm = sizeof(T) == 4 ? (CLS == 0 ? 4 : CLS == 1 ? 3 : 2) : (CLS == 0 ? 3 : CLS == 1 ? 2 : 1);
+  static constexpr int more = sizeof(T) == 4 && CLS < 2 ? per_sm + 1 : per_sm;
 };
 
 // ------------------------------------------------------------ complex lines
@@ -510,7 +516,7 @@ __device__ __forceinline__ void tangle(const TileArgs& a, int t, int k, int N, c
 }
 
 template <typename T, bool PAIR, bool HALF, int CLS>
-__global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_r2c(const __grid_constant__ TileArgs a) {
+__global__ void __launch_bounds__(256, Bounds<T, CLS>::more) k_tile_r2c(const __grid_constant__ TileArgs a) {
   using C = cpx<T>;
   extern __shared__ __align__(16) unsigned char raw[];
   const Tile<C> s = tile_setup<C>(a, raw);
@@ -530,7 +536,7 @@ __global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_r2c(const 
 }
 
 template <typename T, bool PAIR, bool HALF, int CLS>
-__global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_c2r(const __grid_constant__ TileArgs a) {
+__global__ void __launch_bounds__(256, Bounds<T, CLS>::more) k_tile_c2r(const __grid_constant__ TileArgs a) {
   using C = cpx<T>;
   extern __shared__ __align__(16) unsigned char raw[];
   if (energy_cta(a)) return;
@@ -604,7 +610,7 @@ __device__ __forceinline__ int n_pos(const TileArgs& a, int m) {
 }
 
 template <typename T, int DIR, int CLS>
-__global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_blue_line(const __grid_constant__ TileArgs a) {
+__global__ void __launch_bounds__(256, Bounds<T, CLS>::more) k_blue_line(const __grid_constant__ TileArgs a) {
   using C = cpx<T>;
   extern __shared__ __align__(16) unsigned char raw[];
   const Tile<C> s = tile_setup<C>(a, raw);
@@ -634,7 +640,7 @@ __global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_blue_line(const
 // |X|^2 = |v|^2 in the energy; the final step of the first and the first step of the
 // second share their elements.
 template <typename T, int CLS>
-__global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_blue_conv(const __grid_constant__ TileArgs a) {
+__global__ void __launch_bounds__(256, Bounds<T, CLS>::more) k_blue_conv(const __grid_constant__ TileArgs a) {
   using C = cpx<T>;
   extern __shared__ __align__(16) unsigned char raw[];
   __shared__ T wsum[8];
@@ -716,7 +722,7 @@ __global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_blue_conv(const
 }
 
 template <typename T, bool PAIR, int CLS>
-__global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_blue_r2c(const __grid_constant__ TileArgs a) {
+__global__ void __launch_bounds__(256, Bounds<T, CLS>::more) k_blue_r2c(const __grid_constant__ TileArgs a) {
   using C = cpx<T>;
   extern __shared__ __align__(16) unsigned char raw[];
   const Tile<C> s = tile_setup<C>(a, raw);
@@ -740,7 +746,7 @@ __global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_blue_r2c(const 
 }
 
 template <typename T, bool PAIR, int CLS>
-__global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_blue_c2r(const __grid_constant__ TileArgs a) {
+__global__ void __launch_bounds__(256, Bounds<T, CLS>::more) k_blue_c2r(const __grid_constant__ TileArgs a) {
   using C = cpx<T>;
   extern __shared__ __align__(16) unsigned char raw[];
   if (energy_cta(a)) return;
