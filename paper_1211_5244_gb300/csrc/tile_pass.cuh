@@ -318,11 +318,47 @@ __global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_line(const
 
 // ------------------------------------------------------------ forward, K^F, inverse
 
+// The energy of a fused pass: a thread's value (its own lines' terms, in the plan's type)
+// joins the others in 64 bits, across the warp here, across the warps after the next
+// barrier, across the CTAs in the last pass (energy_total). FP32 values cross the warp as
+// sums and their exact errors (Knuth's two-sum), 48 bits: as FP64 additions the five steps
+// hold the two-lane pipe for 80 cycles a warp, with the CTA's barrier behind them (100 x 90 x
+// 110 free, a solve: 32-bit sums 61.0 us, FP64 61.7, two-sums level with 32 bits;
+// 128^3 ffp 62.6, 63.4 and +0.4 us).
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+__device__ __forceinline__ double warp_sum(float v) {
+  float hi = v, lo = 0.f;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float b = __shfl_xor_sync(0xffffffffu, hi, o), l = __shfl_xor_sync(0xffffffffu, lo, o);
+    const float s = hi + b, t = s - hi;
+    lo = (lo + l) + ((hi - (s - t)) + (b - t));
+    hi = s;
+  }
+  // a sum beyond FP32's range, an infinity or a NaN (the same in every lane)
+  if (!(fabsf(hi) <= 3.4028234e38f)) return warp_sum((double)v);
+  return (double)hi + (double)lo;
+}
+template <typename T>
+__device__ __forceinline__ void energy_lanes(T en, double* wsum) {
+  const double v = warp_sum(en);
+  if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = v;
+}
+__device__ __forceinline__ void energy_cta_sum(const TileArgs& a, const double* wsum) {
+  double sum = 0.0;
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) sum += wsum[w];
+  a.partials[blockIdx.y * gridDim.x + blockIdx.x] = sum;
+}
+
 template <typename T, bool HALF, int CLS>
 __global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_conv(const __grid_constant__ TileArgs a) {
   using C = cpx<T>;
   extern __shared__ __align__(16) unsigned char raw[];
-  __shared__ T wsum[8];
+  __shared__ double wsum[8];
   const Tile<C> s = tile_setup<C>(a, raw);
   auto at = [&](int t, int* line, int* pl) {
     const bool ok = line_of(a, t, line, pl);
@@ -381,17 +417,9 @@ __global__ void __launch_bounds__(256, Bounds<T, CLS>::per_sm) k_tile_conv(const
       for (int r = 0; r < R; ++r) p[r * a.es] = x[r];
     });
   });
-  if (a.E != nullptr) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) en += __shfl_xor_sync(0xffffffffu, en, o);
-    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = en;
-  }
+  if (a.E != nullptr) energy_lanes(en, wsum);
   __syncthreads();
-  if (a.E != nullptr && threadIdx.x == 0) {  // the CTA's partial (energy_total adds them in the last pass)
-    double sum = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) sum += (double)wsum[w];
-    a.partials[blockIdx.y * gridDim.x + blockIdx.x] = sum;
-  }
+  if (a.E != nullptr && threadIdx.x == 0) energy_cta_sum(a, wsum);
   step_middle<1, CLS>(a, s);
   step_final<HALF, CLS>(a, s, [&](int t) {
     bool ok;
@@ -643,7 +671,7 @@ template <typename T, int CLS>
 __global__ void __launch_bounds__(256, Bounds<T, CLS>::more) k_blue_conv(const __grid_constant__ TileArgs a) {
   using C = cpx<T>;
   extern __shared__ __align__(16) unsigned char raw[];
-  __shared__ T wsum[8];
+  __shared__ double wsum[8];
   const Tile<C> s = tile_setup<C>(a, raw);
   auto at = [&](int t, int* line, int* pl) {
     const bool ok = line_of(a, t, line, pl);
@@ -698,17 +726,9 @@ __global__ void __launch_bounds__(256, Bounds<T, CLS>::more) k_blue_conv(const _
       });
     }
   });
-  if (a.E != nullptr) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) en += __shfl_xor_sync(0xffffffffu, en, o);
-    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = en;
-  }
+  if (a.E != nullptr) energy_lanes(en, wsum);
   __syncthreads();
-  if (a.E != nullptr && threadIdx.x == 0) {
-    double sum = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) sum += (double)wsum[w];
-    a.partials[blockIdx.y * gridDim.x + blockIdx.x] = sum;
-  }
+  if (a.E != nullptr && threadIdx.x == 0) energy_cta_sum(a, wsum);
   step_middle<-1, CLS>(a, s);
   blue_multiply<1, CLS>(a, s);
   step_middle<1, CLS>(a, s);
