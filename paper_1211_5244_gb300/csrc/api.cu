@@ -459,9 +459,9 @@ int ps_kernel_build(ps_plan p, void* stream) {
       {&p->A, szA, "workspace A"},
       {&p->B, szB, "workspace B"},
       {&p->K, szK, "K^F"},
-      {&p->tw[0], (size_t)p->L[0] * csz, "twiddles x"},
-      {&p->tw[1], (size_t)p->L[1] * csz, "twiddles y"},
-      {&p->tw[2], (size_t)p->L[2] * csz, "twiddles z"},
+      {&p->tw[0], 2 * (size_t)p->L[0] * csz, "twiddles x"},
+      {&p->tw[1], 2 * (size_t)p->L[1] * csz, "twiddles y"},
+      {&p->tw[2], 2 * (size_t)p->L[2] * csz, "twiddles z"},
       {reinterpret_cast<void**>(&p->partials), (size_t)p->npart * sizeof(double), "energy partials"},
       {reinterpret_cast<void**>(&p->counter), 2 * sizeof(unsigned), "energy counter and status"},
       {&p->tctab, p->tctab_floats * sizeof(float), "tensor-core z tables"},
@@ -479,17 +479,19 @@ int ps_kernel_build(ps_plan p, void* stream) {
     }
     total += a.bytes;
   }
+  for (int j = 0; j < 3; ++j) p->twt[j] = static_cast<char*>(p->tw[j]) + p->L[j] * csz;
   for (int j = 0; j < 3 && e == cudaSuccess; ++j) {
     if (!p->blue[j].M) continue;
     const int N = xform_len(p, j);
     void *twM = nullptr, *ch = nullptr, *bf = nullptr;
-    e = cudaMalloc(&twM, (size_t)p->blue[j].M * csz);
+    e = cudaMalloc(&twM, 2 * (size_t)p->blue[j].M * csz);
     if (e == cudaSuccess) e = cudaMalloc(&ch, (size_t)N * csz);
     if (e == cudaSuccess) e = cudaMalloc(&bf, (size_t)p->blue[j].M * csz);
     p->blue[j].twM = twM;
+    p->blue[j].twMt = twM ? static_cast<char*>(twM) + (size_t)p->blue[j].M * csz : nullptr;
     p->blue[j].chirp = ch;
     p->blue[j].Bf = bf;
-    total += (size_t)(2 * p->blue[j].M + N) * csz;
+    total += (size_t)(3 * p->blue[j].M + N) * csz;
   }
   if (e != cudaSuccess) {
     free_device(p);

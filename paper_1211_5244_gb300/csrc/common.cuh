@@ -69,6 +69,7 @@ struct BlueArgs {
   int M;              // 0: the transform runs as plain Stockham stages
   Stages st;          // stages of the length-M transforms
   const void* twM;    // W_M^k, k < M
+  const void* twMt;   // the same as (cos, tan), behind it
   const void* chirp;  // c[m] = exp(-i pi m^2 / N), m < N
   const void* Bf;     // DFT_M of the conjugate chirp, divided by M
 };
@@ -152,6 +153,7 @@ struct ps_plan_s {
   void* B;       // [n3][L2][ldc] complex: y-transformed planes (passes 2..4)
   void* K;       // [H3+1][H2+1][ldk] real: K^F / (L1 L2 L3), even octant (kx < c used)
   void* tw[3];   // W_{L_j}^k, k < L_j, complex, per axis
+  void* twt[3];  // the same as (cos, tan) (tile_dft.cuh), behind tw
   void* tw4z;    // paired z twiddles of the packed z kernel (T*T float4), or NULL
   void* tw4y;    // paired y twiddles of the packed y kernels (16*16 float4), or NULL
   void* twx;     // x passes: W_M^{r c}, r, c < xP (float2, M = L1/2), or NULL

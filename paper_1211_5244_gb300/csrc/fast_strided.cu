@@ -28,17 +28,19 @@ using tile::full_mask;
 
 // The four transforms of a line: columns b forward (P points over a, then the twiddles
 // W_L^{b k1}), rows k1 forward and inverse (Q points), columns inverse (the
-// conjugate twiddles, then P points). At L = 1024 the twiddles are folded into the
-// radix-2 layers of the transform that follows them (480 operations for 32 points behind
-// twiddles instead of about 570; the z pass at 512^3 2202 -> 2158 us, the inverse y
-// pass 579 -> 564 us); the shorter lengths gain no time by it and keep the
-// separate products, whose rounding error is a little smaller.
-template <int P, int Q>
-constexpr bool kFold = P * Q >= 1024;
+// conjugate twiddles, then P points). FOLD (fft_fast.cuh: the z pass and the inverse y pass at
+// L = 1024): the twiddles are folded into the radix-2 layers of the transform that follows
+// them (480 operations for 32 points behind twiddles instead of about 570; the z pass at
+// 512^3 2202 -> 2158 us, the inverse y pass 579 -> 564 us), on the table of (cos, tan) pairs, at a
+// rounding error below that of separate products (32 x 16 x 1024 periodic, round trip of a
+// solve: separate 2.45e-7, folded 2.04e-7). The forward y pass spills 28 bytes in that form
+// (581 -> 620 us), and the shorter lengths gain no time by it.
+template <int P, int Q, int KIND>
+constexpr bool kFold = folded_twiddles(P * Q, KIND);
 
-template <int P, int Q, bool HALF>
+template <int P, int Q, bool HALF, bool FOLD>
 __device__ __forceinline__ void col_fwd(float2 (&y)[P], const float2* tw, int b) {
-  if constexpr (kFold<P, Q>) {
+  if constexpr (FOLD) {
     dft<P, -1, full_mask(HALF ? P / 2 : P)>(y);
   } else {
     rdft<P, -1, HALF>(y);
@@ -46,14 +48,14 @@ __device__ __forceinline__ void col_fwd(float2 (&y)[P], const float2* tw, int b)
     for (int k1 = 1; k1 < P; ++k1) y[k1] = cmul(y[k1], tw[b * k1]);
   }
 }
-template <int P, int Q>
+template <int P, int Q, bool FOLD>
 __device__ __forceinline__ void row_fwd(float2 (&x)[Q], const float2* tw, int k1) {
-  if constexpr (kFold<P, Q>) dft_pre<Q, -1>(x, tw, k1, P);
+  if constexpr (FOLD) dft_pre<Q, -1>(x, tw, k1, P);
   else rdft<Q, -1, false>(x);
 }
-template <int P, int Q>
+template <int P, int Q, bool FOLD>
 __device__ __forceinline__ void row_inv(float2 (&x)[Q], const float2* tw, int k1) {
-  if constexpr (kFold<P, Q>) {
+  if constexpr (FOLD) {
     dft<Q, 1, full_mask(Q)>(x);
   } else {
     rdft<Q, 1, false>(x);
@@ -61,9 +63,9 @@ __device__ __forceinline__ void row_inv(float2 (&x)[Q], const float2* tw, int k1
     for (int b = 1; b < Q; ++b) x[b] = cmulc(x[b], tw[b * k1]);
   }
 }
-template <int P, int Q>
+template <int P, int Q, bool FOLD>
 __device__ __forceinline__ void col_inv(float2 (&y)[P], const float2* tw, int b) {
-  if constexpr (kFold<P, Q>) dft_pre<P, 1>(y, tw, b, Q);
+  if constexpr (FOLD) dft_pre<P, 1>(y, tw, b, Q);
   else rdft<P, 1, false>(y);
 }
 
@@ -110,7 +112,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q),
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
       const int b = j + T * u;
-      col_fwd<P, Q, HALF>(y[u], tw, b);
+      col_fwd<P, Q, HALF, kFold<P, Q, KIND>>(y[u], tw, b);
 #pragma unroll
       for (int k1 = 0; k1 < P; ++k1) sh[(b * P + k1) * TK + t] = y[u][k1];
     }
@@ -120,7 +122,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q),
       const int k1 = j + T * v;
 #pragma unroll
       for (int b = 0; b < Q; ++b) X[v][b] = sh[(b * P + k1) * TK + t];
-      row_fwd<P, Q>(X[v], tw, k1);
+      row_fwd<P, Q, kFold<P, Q, KIND>>(X[v], tw, k1);
     }
   } else {
 #pragma unroll
@@ -167,7 +169,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q),
     // inverse: Q-point transforms over k2, exchange, conjugate twiddles and
     // P-point transforms over k1
 #pragma unroll
-    for (int v = 0; v < NK; ++v) row_inv<P, Q>(X[v], tw, j + T * v);
+    for (int v = 0; v < NK; ++v) row_inv<P, Q, kFold<P, Q, KIND>>(X[v], tw, j + T * v);
     // (KIND 2: back to the slots this thread read its rows from, no barrier before)
 #pragma unroll
     for (int v = 0; v < NK; ++v) {
@@ -182,7 +184,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q),
       float2 y[P];
 #pragma unroll
       for (int k1 = 0; k1 < P; ++k1) y[k1] = sh[(b * P + k1) * TK + t];
-      col_inv<P, Q>(y, tw, b);
+      col_inv<P, Q, kFold<P, Q, KIND>>(y, tw, b);
       if (valid) {
 #pragma unroll
         for (int aa = 0; aa < NA; ++aa)
@@ -344,7 +346,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
       const int b = j + T * u;
-      col_fwd<P, Q, HALF>(y[u], tws, b);
+      col_fwd<P, Q, HALF, kFold<P, Q, 2>>(y[u], tws, b);
 #pragma unroll
       for (int k1 = 0; k1 < P; ++k1) sh[(b * PP + k1) * TK + t] = y[u][k1];
     }
@@ -356,7 +358,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
       const int k1 = j + T * v;
 #pragma unroll
       for (int b = 0; b < Q; ++b) X[v][b] = sh[(b * PP + k1) * TK + t];
-      row_fwd<P, Q>(X[v], tws, k1);
+      row_fwd<P, Q, kFold<P, Q, 2>>(X[v], tws, k1);
       // V^F = K^F rho^F on the even octant of K^F; energy sum K |rho^F|^2
 #pragma unroll
       for (int k2 = 0; k2 < Q; ++k2) {
@@ -367,7 +369,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
         e1 = fmaf(kk, x.x * x.x + x.y * x.y, e1);
         X[v][k2] = make_float2(kk * x.x, kk * x.y);
       }
-      row_inv<P, Q>(X[v], tws, k1);
+      row_inv<P, Q, kFold<P, Q, 2>>(X[v], tws, k1);
     }
     eacc += e1 * ((kx == 0 || 2 * kx == a.L1) ? 1.f : 2.f);
     // back to the slots this thread read its rows from: no barrier before
@@ -392,7 +394,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
       const int b = j + T * u;
-      col_inv<P, Q>(y[u], tws, b);
+      col_inv<P, Q, kFold<P, Q, 2>>(y[u], tws, b);
       if (valid) {
 #pragma unroll
         for (int aa = 0; aa < NA; ++aa)
@@ -546,7 +548,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
 #pragma unroll
       for (int u = 0; u < NB; ++u) {
         const int b = j + T * u;
-        col_fwd<P, Q, HALF>(y[u], tw, b);
+        col_fwd<P, Q, HALF, kFold<P, Q, KIND>>(y[u], tw, b);
 #pragma unroll
         for (int k1 = 0; k1 < P; ++k1) sh[(b * PP + k1) * TK + t] = y[u][k1];
       }
@@ -563,7 +565,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
 #pragma unroll
       for (int v = 0; v < NK; ++v) {
         const int k1 = j + T * v;
-        row_fwd<P, Q>(X[v], tw, k1);
+        row_fwd<P, Q, kFold<P, Q, KIND>>(X[v], tw, k1);
         if (valid) {
 #pragma unroll
           for (int k2 = 0; k2 < Q; ++k2) d[(long long)(k1 + P * k2) * a.dst_elem] = X[v][k2];
@@ -581,7 +583,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
 #pragma unroll
       for (int v = 0; v < NK; ++v) {
         const int k1 = j + T * v;
-        row_inv<P, Q>(X[v], tw, k1);
+        row_inv<P, Q, kFold<P, Q, KIND>>(X[v], tw, k1);
 #pragma unroll
         for (int b = 0; b < Q; ++b) sh[(b * PP + k1) * TK + t] = X[v][b];
       }
@@ -599,7 +601,7 @@ __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (
 #pragma unroll
       for (int u = 0; u < NB; ++u) {
         const int b = j + T * u;
-        col_inv<P, Q>(y[u], tw, b);
+        col_inv<P, Q, kFold<P, Q, KIND>>(y[u], tw, b);
         if (valid) {
 #pragma unroll
           for (int aa = 0; aa < NA; ++aa)

@@ -619,6 +619,13 @@ bool pdl_launches() {
 
 namespace {
 
+// the table of W_L^k that a specialised kernel without one of its own reads
+const void* pass_table(const ps_plan_s* p, int pass) {
+  const int axis = pass_axis(p, pass);
+  const bool folded = (pass == P3 && folded_twiddles(p->L[axis], 2)) || (pass == P4 && folded_twiddles(p->L[axis], 1));
+  return folded ? p->twt[axis] : p->tw[axis];
+}
+
 // One launch of a specialised kernel: programmatic stream serialisation
 // (the kernel may start while the previous one drains; it waits for it before
 // touching memory; PS_PDL=0 off) and, for cluster kernels, the cluster shape.
@@ -704,20 +711,18 @@ cudaError_t launch_fast_chunk(ps_plan_s* p, int pass, const void* rhoV, void* B,
     cf.grid = dim3((unsigned)std::min<long long>(cf.grid.x, tiles));
   }
   const float* K = static_cast<const float*>((pass == P1 || pass == P5) ? p->twx : p->K);
-  const int axis = pass_axis(p, pass);
-  const void* tw = ((pass == P2 && (p->ysoa & 1)) || (pass == P4 && (p->ysoa & 2))) ? p->tw4y : p->tw[axis];
+  const void* tw = ((pass == P2 && (p->ysoa & 1)) || (pass == P4 && (p->ysoa & 2))) ? p->tw4y : pass_table(p, pass);
   return launch_cfg(cf, fa, src, dst, K, tw, p->partials, p->counter, escale, E, s);
 }
 
 cudaError_t launch_fast(ps_plan_s* p, int pass, const void* src, void* dst, double* E, double escale,
                         cudaStream_t s, VjpTerm* add) {
   PassCfg cf = p->cfg[pass];
-  const int axis = pass_axis(p, pass);
   // x passes get the twiddle matrix in the K slot
   const float* K = static_cast<const float*>((pass == P1 || pass == P5) ? p->twx : p->K);
   const void* tw = (pass == P3 && p->tctab) ? p->tctab
                    : (pass == P3 && p->zsoa_T) ? p->tw4z
-                   : ((pass == P2 && (p->ysoa & 1)) || (pass == P4 && (p->ysoa & 2))) ? p->tw4y : p->tw[axis];
+                   : ((pass == P2 && (p->ysoa & 1)) || (pass == P4 && (p->ysoa & 2))) ? p->tw4y : pass_table(p, pass);
   FastArgs fa = cf.fa;
   fa.nparts = z_pass_ctas(p);
   if (pass == P5 && add != nullptr) {

@@ -55,6 +55,9 @@ using FastKernel = void (*)(const void*, void*, const float*, const float2*, Fas
 //   kind 0: forward (n nonzero inputs, L outputs), 1: inverse (L inputs,
 //   n outputs), 2: forward, K^F multiply, inverse; half: n = L/2 (else n = L)
 const void* strided_kernel(int L, int kind, bool half, int* threads, size_t* smem, int* tk);
+// Whether an unpacked y or z kernel (kind as above) folds its twiddles into its transforms (dft_pre,
+// tile_dft.cuh; the measurements are at col_fwd): it takes the table of (cos, tan) pairs, p->twt.
+constexpr bool folded_twiddles(int L, int kind) { return L >= 1024 && kind != 0; }
 // Returns the kernel for an x pass (real length 2M): kind 0 R2C, 1 C2R, 2 C2R that adds the
 // energy term of a vector-Jacobian product.
 const void* xline_kernel(int M, int kind, bool half, int* threads, int* rows, size_t* smem);

@@ -25,6 +25,7 @@
 #include <cmath>
 
 #include "common.cuh"
+#include "tile_dft.cuh"
 
 namespace ps {
 
@@ -211,11 +212,12 @@ __global__ void store_kernel(const double* __restrict__ M, T* __restrict__ K, si
 }
 
 template <typename T>
-__global__ void twiddle_kernel(cpx<T>* tw, int L) {
+__global__ void twiddle_kernel(cpx<T>* tw, cpx<T>* twt, int L) {
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < L; k += gridDim.x * blockDim.x) {
     double s, c;
     sincospi(2.0 * k / L, &s, &c);
     tw[k] = mk((T)c, (T)(-s));
+    twt[k] = tile::tan_pair<T>(k, L);
   }
 }
 
@@ -244,19 +246,20 @@ __global__ void twiddle_pairs_kernel(float4* tw4, int L, int T, int P) {
 // Bluestein tables for a transform of length N, convolution length M:
 //   chirp[m] = exp(-i pi m^2 / N), m < N
 //   Bf[k] = (1/M) sum_j b[j] W_M^{jk}, b[j] = conj(chirp[|j|]) for |j| < N (j taken mod M)
-// Phases are reduced exactly in integers (m^2 mod 2N, j k mod M) before sincospi.
+// Phases are reduced exactly in integers (m^2 mod 2N, j k mod M) before the sines and
+// cosines. In FP64 an error of B's table stands in every line's result, forward and
+// inverse: its terms 2 cos(2 pi j k / M) exp(+i pi j^2 / N) come from the rounded tables
+// (the cosines of twMt, the chirp) and are added with their rounding errors, where
+// sincospi of a - w in doubles was off by the rounding of angles up to 4 pi, and the sum by
+// that of N additions (37^3 periodic, round trip of a solve: 1.25e-15 -> 6.4e-16).
 template <typename T>
 __global__ void chirp_kernel(cpx<T>* ch, int N) {
   for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < N; m += gridDim.x * blockDim.x) {
-    const long long q = ((long long)m * m) % (2LL * N);
-    double s, c;
-    sincospi((double)q / N, &s, &c);
-    ch[m] = mk((T)c, (T)(-s));
+    ch[m] = tile::turn<T>((long)(((long long)m * m) % (2LL * N)), 2L * N);
   }
 }
 
-template <typename T>
-__global__ void bluestein_bf_kernel(cpx<T>* Bf, int N, int M) {
+__global__ void bluestein_bf_kernel(float2* Bf, int N, int M) {
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < M; k += gridDim.x * blockDim.x) {
     double re = 0.0, im = 0.0;
     for (int j = 0; j < N; ++j) {
@@ -272,7 +275,25 @@ __global__ void bluestein_bf_kernel(cpx<T>* Bf, int N, int M) {
         im += s;
       }
     }
-    Bf[k] = mk((T)(re / M), (T)(im / M));
+    Bf[k] = mk((float)(re / M), (float)(im / M));
+  }
+}
+
+__global__ void bluestein_bf_kernel(double2* Bf, const double2* chirp, const double2* twMt, int N, int M) {
+  // (hi, lo) += v with the addition's error (Knuth's two-sum)
+  auto add = [](double& hi, double& lo, double v) {
+    const double s = __dadd_rn(hi, v), t = __dadd_rn(s, -hi);
+    lo += __dadd_rn(__dadd_rn(hi, -__dadd_rn(s, -t)), __dadd_rn(v, -t));
+    hi = s;
+  };
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < M; k += gridDim.x * blockDim.x) {
+    double re = 1.0, im = 0.0, rl = 0.0, il = 0.0;
+    for (int j = 1; j < N; ++j) {
+      const double c = 2.0 * twMt[((long long)j * k) % M].x;
+      add(re, rl, c * chirp[j].x);
+      add(im, il, -c * chirp[j].y);
+    }
+    Bf[k] = mk((re + rl) / M, (im + il) / M);
   }
 }
 
@@ -288,22 +309,23 @@ cudaError_t build_twiddles(ps_plan_s* p, cudaStream_t s) {
   for (int j = 0; j < 3; ++j) {
     const int L = p->L[j];
     if (p->dtype == PS_F32)
-      twiddle_kernel<float><<<grid_for(L), 256, 0, s>>>(static_cast<float2*>(p->tw[j]), L);
+      twiddle_kernel<float><<<grid_for(L), 256, 0, s>>>(static_cast<float2*>(p->tw[j]), static_cast<float2*>(p->twt[j]), L);
     else
-      twiddle_kernel<double><<<grid_for(L), 256, 0, s>>>(static_cast<double2*>(p->tw[j]), L);
+      twiddle_kernel<double><<<grid_for(L), 256, 0, s>>>(static_cast<double2*>(p->tw[j]), static_cast<double2*>(p->twt[j]), L);
   }
   for (int j = 0; j < 3; ++j) {
     const BlueArgs& b = p->blue[j];
     if (!b.M) continue;
     const int N = xform_len(p, j);
     if (p->dtype == PS_F32) {
-      twiddle_kernel<float><<<grid_for(b.M), 256, 0, s>>>((float2*)b.twM, b.M);
+      twiddle_kernel<float><<<grid_for(b.M), 256, 0, s>>>((float2*)b.twM, (float2*)b.twMt, b.M);
       chirp_kernel<float><<<grid_for(N), 256, 0, s>>>((float2*)b.chirp, N);
-      bluestein_bf_kernel<float><<<grid_for(b.M), 256, 0, s>>>((float2*)b.Bf, N, b.M);
+      bluestein_bf_kernel<<<grid_for(b.M), 256, 0, s>>>((float2*)b.Bf, N, b.M);
     } else {
-      twiddle_kernel<double><<<grid_for(b.M), 256, 0, s>>>((double2*)b.twM, b.M);
+      twiddle_kernel<double><<<grid_for(b.M), 256, 0, s>>>((double2*)b.twM, (double2*)b.twMt, b.M);
       chirp_kernel<double><<<grid_for(N), 256, 0, s>>>((double2*)b.chirp, N);
-      bluestein_bf_kernel<double><<<grid_for(b.M), 256, 0, s>>>((double2*)b.Bf, N, b.M);
+      bluestein_bf_kernel<<<grid_for(b.M), 256, 0, s>>>((double2*)b.Bf, (const double2*)b.chirp, (const double2*)b.twMt,
+                                                        N, b.M);
     }
   }
   if (p->xP)

@@ -16,7 +16,7 @@ struct TileArgs {
   const void* src;
   void* dst;
   const void* K;    // K^F octant (conv)
-  const void* tw;   // W_N^j at tw[j * tws]
+  const void* tw;   // W_N^j at tw[j * tws], as (cos, tan) (tan_pair)
   const void* twL;  // x real passes of even length: W_L^k, L = 2 N
   int tws;
   int N, Ra, Rm, Rl;

@@ -19,7 +19,7 @@
 // passes.cu, which make a shared-memory round trip per stage and more for the load,
 // the multiply and the store, and spend a third of their issue slots on integer
 // instructions), in FP64 the two FP64 lanes per clock and SM (128^3 free: 1657
-// -> 1203 us; the pipe was 84% busy before, so only fewer operations help).
+// -> 1161 us; the pipe was 84% busy before, so only fewer operations help).
 #pragma once
 
 #include "fft_fast.cuh"
