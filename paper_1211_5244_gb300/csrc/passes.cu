@@ -593,11 +593,17 @@ cudaError_t configure_passes(ps_plan_s* p) {
       // x first (x, z, y): the specialised x kernels, and the y- and z-pass
       // kernels along z and y through strides, when all three middle passes have them
       if (p->ord[0] == 0) {
+        const std::vector<PassCfg> strided(p->cfg, p->cfg + 5);
         if ((e = configure_fast_f32(p)) != cudaSuccess) return e;
         p->fastord = p->cfg[P2].fast && p->cfg[P3].fast && p->cfg[P4].fast;
         if (p->fastord) {
           const int ntk = (p->c + p->cfg[P3].tk - 1) / p->cfg[P3].tk;
           p->npart = std::max(p->npart, ntk * p->L[p->ord[1]]);
+        } else {
+          // the strided kernels run every pass, on their own tiles (a z kernel's width in
+          // cfg[P3].tk would overlap their rows or outgrow the energy partials)
+          std::copy(strided.begin(), strided.end(), p->cfg);
+          p->xP = p->ysoa = p->zsoa_T = p->zsoa_P = 0;  // nor are the register kernels' tables read
         }
       }
     }
