@@ -254,9 +254,12 @@ __device__ __forceinline__ void step_inv_first(const TileArgs& a, const Tile<C>&
 
 // Resident CTAs (of 256 threads) per SM asked of the compiler. The FP32 passes are
 // bound by latency, so more warps pay where the radices still fit their registers:
-// the real and the Bluestein passes take one CTA more (64 registers for class 1; 32
-// uneven problems 860 -> 834 us). The fused pass spills there (128^3 ffp 59.3 ->
-// 64.7 us), and the line pass loses by it (100 x 90 x 110 free 62.0 -> 63.0 us).
+// the real passes and the Bluestein form take one CTA more (64 registers for class 1; 32
+// uneven problems 860 -> 834 us). The fused pass spills there (128^3 ffp 59.3 -> 64.7 us),
+// and the line pass loses by it (100 x 90 x 110 free 62.0 -> 63.0 us). The fused Bluestein
+// pass spills 96 bytes and loses alone (the z pass of 74 x 79 x 83 free 40.9 -> 43.4 us, of 127 x 131 x
+// 113 periodic 23.0 -> 25.2), but in a batch, where its CTAs share the SMs with other problems', the
+// narrower one gains: 32 uneven problems 853 -> 837 us.
 template <typename T, int CLS>
 struct Bounds {
   static constexpr int per_sm = sizeof(T) == 4 ? (CLS == 0 ? 4 : CLS == 1 ? 3 : 2) : (CLS == 0 ? 3 : CLS == 1 ? 2 : 1);
