@@ -193,7 +193,9 @@ int ps_plan_set_order(ps_plan plan, int a0, int a1, int a2);
  * `stream` (reps < 1 means 5); the choice is set on `plan` (not built; see
  * ps_plan_info.schedule). Results are cached per geometry and device in
  * memory and, when the environment variable PS_TUNE_CACHE names a file, in
- * that file. Must precede ps_kernel_build; synchronises `stream`.
+ * that file (lines of an earlier format, tuned on other kernels, are not
+ * used; the geometry is tuned again). Must precede ps_kernel_build;
+ * synchronises `stream`.
  * Errors: PS_ERR_ARG (plan NULL or built), PS_ERR_OOM, PS_ERR_CUDA.
  */
 int ps_plan_autotune(ps_plan plan, int reps, void* stream);

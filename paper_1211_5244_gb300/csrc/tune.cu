@@ -25,8 +25,10 @@
 // Results are kept in memory, and in a text file when PS_TUNE_CACHE names one
 // (one line per geometry: "n1 n2 n3 bc1 bc2 bc3 mode sms L1 L2 L3 tile radix
 // ztk ykind xy xfirst chunks tile_x tile_y tile_z radix_x+1 radix_y+1
-// radix_z+1", mode = dtype + 2 math + 4 (the plan's order as 9 a0 + 3 a1 +
-// a2), 0 for a default choice).
+// radix_z+1 format", mode = dtype + 2 math + 4 (the plan's order as 9 a0 + 3 a1 +
+// a2), 0 for a default choice, format = kFormat). Lines without the format, or with
+// another, are left in the file and not used: they were timed on other kernels (before the
+// tile kernels, radix 1 only chose among Stockham stages), so the geometry is tuned again.
 #include <algorithm>
 #include <cstdio>
 #include <cstdlib>
@@ -44,6 +46,10 @@ namespace {
 // a tuned choice: padded lengths and the schedule fields of the plan
 enum { kL1, kL2, kL3, kTile, kRadix, kZtk, kYkind, kXy, kXfirst, kChunks, kTileAx, kRadixAx = kTileAx + 3,
        kFields = kRadixAx + 3 };
+
+// what the choices of a line in the file stand for; another number whenever a field comes to mean
+// other kernels
+constexpr int kFormat = 2;
 
 std::mutex g_tune_mu;
 std::map<std::string, std::vector<int>> g_tuned;
@@ -70,7 +76,7 @@ void load_file() {
   if (!f) return;
   char line[512];
   while (fgets(line, sizeof line, f)) {
-    // 8 key fields, then the choice; lines of another field count are skipped
+    // 8 key fields, the choice, the format; other lines are skipped
     std::vector<long> w;
     char* q = line;
     while (true) {
@@ -80,10 +86,10 @@ void load_file() {
       w.push_back(x);
       q = end;
     }
-    if (w.size() != (size_t)(8 + kFields)) continue;
+    if (w.size() != (size_t)(8 + kFields + 1) || w.back() != kFormat) continue;
     char key[128];
     snprintf(key, sizeof key, "%ld %ld %ld %ld %ld %ld %ld %ld", w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
-    g_tuned[key] = std::vector<int>(w.begin() + 8, w.end());
+    g_tuned[key] = std::vector<int>(w.begin() + 8, w.end() - 1);
   }
   fclose(f);
 }
@@ -95,7 +101,7 @@ void append_file(const std::string& key, const std::vector<int>& v) {
   if (!f) return;
   fprintf(f, "%s", key.c_str());
   for (int x : v) fprintf(f, " %d", x);
-  fprintf(f, "\n");
+  fprintf(f, " %d\n", kFormat);
   fclose(f);
 }
 
