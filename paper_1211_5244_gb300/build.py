@@ -3,6 +3,12 @@
 Each .cu file is compiled to an object in parallel, then linked into
 ``paper_1211_5244_gb300/lib/libpsolver.so``. A build is skipped when the
 library is newer than every source and header.
+
+The ten tile_*.cu files are most of the work: 80 to 140 CPU seconds each in the compiler's
+optimiser, for a body per radix up to 16, step, direction and kind of pass. A clean build takes
+212 s on 8 x86 cores and 65 s on 16 Grace cores (41 s and 26 s without the tile kernels). Starting
+them first gains nothing; nvcc's fast compilation (-Ofc min) takes a third of the time, and the
+FP32 kernels it makes are 12 to 20% slower.
 """
 from __future__ import annotations
 

@@ -230,7 +230,9 @@ const void* strided_kernel(int L, int kind, bool half, int* threads, size_t* sme
 // = (kx tile, ky row in the paired order) with kx fastest. The tile's n3 input
 // rows land in the exchange (cp.async), the K^F octant slice in a stage of its
 // own; the next tile's K^F slice is copied once the current one has been
-// used, its input rows once the exchange has been read for the last time.
+// used (after a CTA barrier), its input rows once the warp has read the exchange for the
+// last time: a warp copies the rows that its own threads read, into slots that
+// only they write.
 // With 8 lines per tile (64-byte exchange rows) the exchange has one padding
 // row after every 32: the four line positions j of a warp then write rows 33
 // apart, on alternate halves of the banks, instead of 32 apart on the same
@@ -445,8 +447,12 @@ const void* zpipe_u_kernel(int L, bool half, int* threads, size_t* smem, int* tk
 // stores of the current tile run. With 8 lines per tile (64-byte rows) the
 // exchange has one padding row after every 32, as in the L = 1024 z kernel:
 // the forward write and the inverse read of a warp then fall on alternate
-// bank halves instead of 4-way on the same 16 banks. The input rows keep the
-// unpadded layout (they are read before the exchange is written).
+// bank halves instead of 4-way on the same 16 banks. The input rows land in the
+// exchange's own (padded) slots: forward, row b + Q aa in (b, aa), inverse, row k1 + P k2
+// in (k2, k1). A warp copies exactly the rows that its threads read, and overwrites
+// exactly their slots with its half of the exchange, so __syncwarp orders the copy, the
+// reads and the writes; the exchange is then read across the warps, between two CTA
+// barriers, the second before the next tile's copies.
 template <int P, int Q, int KIND, bool HALF, int TK>
 __global__ void __launch_bounds__(TK*(P < Q ? P : Q), P > Q ? 512 / (TK * Q) : (P * Q >= 512 ? 2 : 3))
     k_ypipe(const void* src_v, void* dst_v, const float*, const float2* __restrict__ tw, FastArgs a, double*,

@@ -49,8 +49,10 @@ __device__ inline void energy_finish(double part, double* partials, unsigned* co
 }
 
 // The energy of a solve in two halves. The z pass (or the fused pass along
-// another axis) stores one partial per CTA and is done; CTA 0 of the last pass
-// adds them in index order after its own work, beside the other CTAs. A
+// another axis) stores one partial per CTA and is done; one CTA of the last pass adds them
+// in a fixed order (four strided sums per thread, then the CTA's sum: the same
+// partials give the same bits), beside the other CTAs: CTA 0 after its own rows in
+// the register and Stockham kernels, one without lines of its own in the tile kernels. A
 // last-arriving CTA in the z pass itself cost its fence, its atomic and the sum at
 // the end of the pass, where nothing else runs (128^3 wire FP32: 40.8 us per solve
 // against 37.1 without the energy).

@@ -1,8 +1,13 @@
-// Tile kernels: the passes of a solve for any line length with factors up to
-// 13, FP32 and FP64, along any axis, as two (or three) register DFT steps with
-// one exchange through shared memory between them.
+// Tile kernels: the passes of a solve for a line of any length that tile_radix
+// (tile_launch.cu) factors, FP32 and FP64, along any axis, as two (or three) register
+// DFT steps with one exchange through shared memory between them. It factors products of
+// two or three radices up to 16, and a prime from 17 to 31 behind at most two of them;
+// other lengths with a prime factor from 11 on run in Bluestein form (below). Smooth
+// lengths that need a fourth radix (48 from 625 on: 625, 875, 1250, 2000, 2187, 4000, ...)
+// and 2, 3, 5 and 7 stay on the Stockham kernels.
 //
-// A CTA owns a tile of tk lines; T threads share a line. With
+// A CTA owns a tile of tk lines; the butterflies of a step are spread over its threads
+// (tasks). With
 // N = Ra Rm Rl, n = n1 NRa + n2 Rl + n3 and k = k1 + Ra k2 + Ra Rm k3 the forward
 // transform is
 //   first  (n2, n3): Ra-point DFT over n1 -> k1, inputs straight from global memory
@@ -594,7 +599,8 @@ __global__ void __launch_bounds__(256, Bounds<T, CLS>::more) k_tile_c2r(const __
 
 // ------------------------------------------------------------ Bluestein form
 
-// Lines whose length N has a prime factor above 31 (or two above 16): the chirp-z
+// Lines whose length N has a prime factor from 11 on and no factorisation into steps (a
+// prime above 31, two above 16, or 11 and 13 themselves): the chirp-z
 // form X[k] = c[k] sum_m (x[m] c[m]) conj(c[k-m]), c[m] = exp(-i pi m^2 / N), as a
 // cyclic convolution of length M >= 2 N on the steps above (a.N = M, a.Nt = N):
 // the chirp product in the loads, the product with the transformed conjugate chirp Bf
