@@ -132,7 +132,8 @@ __device__ inline cpx<T> turn(long j, long N) {
 }
 // W_N^j = exp(-2 pi i j / N) as (c, t), W = c (1 + i t): the form of the tables behind dft_pre (see bfly_w,
 // mul_t). t is of the rounded c, so that c t is the sine to one rounding; where the cosine
-// is 0 a c far below the type's last bit of 1 stands for it.
+// is 0 a c far below the type's last bit of 1 stands for it (its product with t overflows for
+// FP32 values from 2^100 on, FP64 from 2^964).
 template <typename T>
 __device__ inline cpx<T> tan_pair(int j, int N) {
   const bool zero = 4 * j == N || 4 * j == 3 * N;

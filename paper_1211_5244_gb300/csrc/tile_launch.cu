@@ -122,7 +122,9 @@ void tile_axes(int al, int* at, int* ap) {
 // most threads whose last round of butterflies is not emptier by more than a tenth
 // (90 x 75 x 110 ppf, L3 = 220, 450 CTAs: 64 -> 192 threads, solve 32.7 -> 28.5 us).
 // With the line at 768 threads per SM a batch of 32 such problems, which fills the
-// chip, goes from 865 to 894 us; the other passes gain nothing from more threads.
+// chip, goes from 865 to 894 us; the other passes gain nothing from more threads. (A plan
+// does not know whether it runs alone: in a batch the other problems' CTAs fill the SMs, and
+// the line lies between what that grid alone and that batch want.)
 //
 // In FP64 a warp instruction holds the pipe as long with one lane as with 32: the
 // tile is the width with the fewest operations per SM, counting whole warps and
